@@ -73,8 +73,8 @@ def peaks():
         return {"hbm_gbs": 6800.0, "bf16": 1900.0, "bf16_sustained": 1700.0, "source": "fallback"}
 
 
-ATTN_SOURCES = ("paper_2106_06899_gb300/csrc/attn_tc.cu", "paper_2106_06899_gb300/csrc/select.cuh",
-                "paper_2106_06899_gb300/csrc/common.cuh")
+ATTN_SOURCES = ("paper_2106_06899_gb300/csrc/attn_tc.cuh", "paper_2106_06899_gb300/csrc/rowlist.cuh",
+                "paper_2106_06899_gb300/csrc/rowfinish.cuh", "paper_2106_06899_gb300/csrc/common.cuh")
 
 
 def profiled_traffic(w):

@@ -1,0 +1,877 @@
+// attn_tc.cuh -- fused top-k attention (Eq. 4) for bf16 inputs on sm_103a.
+//
+// One persistent CTA per SM walks work units: a unit is RT query tiles of 128
+// rows of one (b, h).  For a unit the query tiles (Sec. 2.2 "Query chunking",
+// C = 128 RT) are loaded once by TMA, then the keys stream through in tiles of
+// N that all RT query tiles share:
+//
+//   warp 0       TMA producer: the query tiles, then K tiles into a ring
+//   warps 1, 2   MMA issuers, one per query tile: S = Q K_tile^T with
+//                tcgen05.mma (bf16 in, fp32 accumulate) into that query tile's
+//                TMEM accumulators [128 x N]
+//   warps 4 ..   filters, four per query tile: lane t of warp w owns TMEM lane
+//                / query row 32 (w % 4) + t.  It reads its scores with
+//                tcgen05.ld.red, which returns each group of eight together
+//                with its maximum, and keeps the row's candidates in its list
+//                (rowlist.cuh).  After the unit's last key tile it cuts the
+//                lists to the exact top k and hands them over.
+//   the rest     epilogue: a warp per row orders the kept keys if the
+//                selection is an output, applies the softmax over them and
+//                gathers the matching value rows (rowfinish.cuh), while the
+//                filters stream the next unit.
+//
+// The score tile never leaves TMEM/registers: no [C x Lk] matrix is written
+// to device memory (Sec. 2.2 "Query chunking": memory O(C Lk) becomes
+// O(C k) here, in shared memory).  The scale of Eq. 1 is folded into Q by
+// the caller.  Causal masking (Eq. 2) skips key tiles past the query tile
+// and masks keys j > i inside the diagonal tile.
+//
+// Every pipeline wait is bounded (common.cuh); on expiry the CTA stops,
+// drains its in-flight copies and MMAs, frees TMEM and returns.
+#pragma once
+
+#include <algorithm>
+#include <type_traits>
+
+#include "kernels.h"
+#include "rowfinish.cuh"
+#include "rowlist.cuh"
+
+namespace topk {
+
+namespace {
+
+constexpr int BM = 128;        // rows of an MMA tile
+constexpr int kThreads = 512;  // 4 control warps, 4 RT filter warps, the rest epilogue
+
+// D: head size; RT: query tiles per unit; RPU: query rows of a tile that
+// belong to the unit.  The MMA tile always has 128 rows; with RPU = 64 or 32
+// (RT = 1) only the first RPU of them are the unit's, so that one row's list
+// can hold several hundred keys.
+template <int D, typename IdxT, int RT, int RPU>
+struct Layout {
+  static_assert(RT == 1 || RPU == BM, "reduced-row units take one query tile");
+  static constexpr int N = D == 64 ? 128 : 64;  // keys per tile: 16 KB of K
+  static constexpr int S = RT == 2 || RPU < BM ? 2 : 3;  // K stages
+  static constexpr int R = D / 64;  // 128-byte column blocks per row
+  // Scores per offer and records per row (rowlist.cuh).  Eight records where
+  // the lists leave room (k = 256: 3.0 ms against 3.5 with four at L = 8192),
+  // four beside two query tiles' lists and at d = 128 (k = 128, L = 16384: 8.9 ms;
+  // eight leave lists so short that they prune all the time: 15.5).
+  static constexpr int OFFER = D == 128 && RPU == BM ? 16 : 32;
+  static constexpr int RECS = RT == 2 || (D == 128 && RPU == BM) ? 4 : 8;
+  using List = RowList<IdxT, RECS>;
+  static constexpr int NQ = RPU / 32;      // filter warps per query tile
+  static constexpr int NJ = RT * NQ;       // filter warps in all
+  static constexpr int NE = 12 - 4 * RT;   // epilogue warps
+  static constexpr int NS = NE > NJ ? NE / NJ : 1;  // epilogue warps that share a filter warp's rows
+  static constexpr int RS = 32 / NS;       // rows each of them takes
+  // The kept lists go through a device buffer of SL slots per filter warp, so
+  // that the epilogue of one unit overlaps the filtering of the next.  Large-k
+  // kernels hand their lists over in place: a unit's filtering is long against
+  // its epilogue there.
+  static constexpr bool kPark = RPU == BM;
+  static constexpr int SL = 4 / RT;  // the same buffer size for both RT
+  static constexpr uint32_t Q_BYTES = BM * D * 2;  // one query tile
+  static constexpr uint32_t KST_BYTES = N * D * 2;
+  static constexpr size_t OFF_Q = 0;
+  static constexpr size_t OFF_K = OFF_Q + static_cast<size_t>(RT) * Q_BYTES;
+  static constexpr size_t OFF_CTRL = OFF_K + static_cast<size_t>(S) * KST_BYTES;
+  // TMEM accumulators per query tile: as many N-column buffers as fit in 512
+  // columns, at most 4, so that the MMAs run ahead of a filter that prunes
+  static constexpr int NACC = 512 / (RT * N) < 4 ? 512 / (RT * N) : 4;
+  static constexpr uint32_t TMEM_COLS = RT * NACC * N;
+  static constexpr int NBARS = 2 * S + 2 + 2 * RT * NACC + RT;
+  static constexpr size_t CTRL_BYTES = (static_cast<size_t>(NBARS) * 8 + 8 + 2 * 8 * 4 + RPU * 4 + 127) & ~size_t(127);
+  // Candidates of a row that the epilogue takes at most: the exact top k is its
+  // work (a warp per row finds it faster than a filter's lockstep passes do).
+  static constexpr int hand(int topk) { return (topk + 32 + 31) & ~31; }
+  static constexpr size_t OFF_LIST = OFF_CTRL + CTRL_BYTES;
+  static constexpr size_t kMaxSmem = 232448;
+  static constexpr size_t kFixed = 1024 + OFF_LIST;
+
+  static constexpr int min_cap(int topk) { return (topk + kListSlack + 8 + 7) & ~7; }
+  // the epilogue warps' buffers, behind the lists
+  static constexpr size_t buf_bytes(int topk) { return static_cast<size_t>(NE) * topk * sizeof(uint2); }
+  // List slots per row: what fits, up to about 2.5 k + 64 (longer lists prune
+  // less often but let their thresholds lag further behind).
+  static int cap(int topk) {
+    const int want = (5 * topk / 2 + 64 + 7) & ~7;
+    int c = static_cast<int>((kMaxSmem - kFixed) / NJ / (kListStride * (4 + sizeof(IdxT)))) & ~7;
+    while (c > 0 && kFixed + buf_bytes(topk) + NJ * List::bytes(c) > kMaxSmem) c -= 8;
+    c = std::min(c, std::max(want, min_cap(topk)));
+    return c >= min_cap(topk) ? c : 0;
+  }
+  static bool fits(int topk) { return cap(topk) > 0; }
+  // Classes of the bound stretch (RowList): 2 k, or what the warp's memory holds.
+  static int classes(int topk) {
+    return std::min((std::max(2 * topk, 16) + 15) & ~15,
+                    static_cast<int>(List::bytes(cap(topk)) / (kListStride * 4)) & ~15);
+  }
+  static size_t bytes(int topk) { return kFixed + buf_bytes(topk) + NJ * List::bytes(cap(topk)); }
+
+  static constexpr size_t park_keys_per_cta(int topk) { return kPark ? static_cast<size_t>(NJ) * SL * 32 * hand(topk) : 0; }
+  static constexpr size_t park_bytes(int grid, int topk) {
+    return kPark ? static_cast<size_t>(grid) * (park_keys_per_cta(topk) * 8 + NJ * SL * 32 * 4) : 0;
+  }
+};
+
+// Waits for an mbarrier phase: every lane tries once, then lane 0 polls.  The
+// whole warp leaves together.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
+                                          volatile int* abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  int ok = 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow(bar, parity, ctl, abort_flag) ? 1 : 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  if (ok) (void)mbar_try_wait(bar, parity);  // every lane observes the completed phase
+  return ok != 0;
+}
+
+// Waits (bounded; lane 0 polls) until the shared-memory counter *ctr, which
+// only grows, reaches target; every lane then reads it with acquire
+// semantics itself, so that what the releasing warp wrote before it is
+// visible to the whole warp.  False if the CTA aborts or the limit runs out.
+__device__ __forceinline__ bool wait_count(uint32_t* ctr, uint32_t target, const DevCtl& ctl,
+                                           volatile int* abort_flag) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0 && static_cast<int>(ld_acquire_u32(ctr) - target) < 0) {
+    const unsigned long long t0 = global_ns();
+    for (uint32_t spin = 0;; ++spin) {
+      if (static_cast<int>(ld_acquire_u32(ctr) - target) >= 0) break;
+      if ((spin & 15u) == 15u) {
+        if (*abort_flag) {
+          ok = 0;
+          break;
+        }
+        if (global_ns() - t0 > ctl.wait_limit_ns) {
+          atomicOr(ctl.error, kDevErrTimeout);
+          *abort_flag = 1;
+          ok = 0;
+          break;
+        }
+      }
+      __nanosleep(32u << (spin < 4u ? spin : 4u));
+    }
+  }
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  if (ok) (void)ld_acquire_u32(ctr);
+  return ok != 0;
+}
+
+// Bounded wait that ignores the abort flag: used only to drain in-flight
+// asynchronous work before the CTA exits.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, const DevCtl& ctl) {
+  const unsigned long long t0 = global_ns();
+  while (!mbar_try_wait(bar, parity)) {
+    if (global_ns() - t0 > ctl.wait_limit_ns) {
+      atomicOr(ctl.error, kDevErrTimeout);
+      return;
+    }
+  }
+}
+
+// Keeps the wait for a tcgen05.ld ahead of every use of what it loaded.
+template <int NV, int NM>
+__device__ __forceinline__ void tmem_wait_tied(float (&v)[NV], float (&m)[NM]) {
+  tmem_wait_ld();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) asm volatile("" : "+f"(v[i]));
+#pragma unroll
+  for (int i = 0; i < NM; ++i) asm volatile("" : "+f"(m[i]));
+}
+
+// 8 G consecutive TMEM columns of this thread's lane and the maxima of their
+// groups of eight.
+template <int G>
+__device__ __forceinline__ void load_chunk(uint32_t taddr, float (&v)[8 * G], float (&m)[G]) {
+#pragma unroll
+  for (int g = 0; g < G; ++g) tmem_ld8_max(taddr + 8 * g, reinterpret_cast<float(&)[8]>(v[8 * g]), m[g]);
+}
+
+template <int D, typename IdxT, int RT, int RPU>
+__global__ void __launch_bounds__(kThreads, 1)
+    attn_tc_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
+                   const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out, int BH, int H, int Lq,
+                   int Lk, int topk, int cap, int classes, int bound_den, int causal, const int32_t* __restrict__ kv_len, int n_units,
+                   int parts, uint2* __restrict__ part_keys, int* __restrict__ part_n, int32_t* __restrict__ idx,
+                   float* __restrict__ score, uint2* __restrict__ park, int* __restrict__ park_n, DevCtl ctl) {
+  using L = Layout<D, IdxT, RT, RPU>;
+  using List = typename L::List;
+  constexpr int kOffer = L::OFFER;
+  constexpr int N = L::N, S = L::S, R = L::R, NACC = L::NACC, NQ = L::NQ, NJ = L::NJ, NE = L::NE;
+  constexpr uint32_t IDESC = idesc_bf16_f32(BM, N);
+  constexpr int RU = RPU * RT;  // query rows per unit
+  const int hand = L::hand(topk);
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint8_t* q_s = smem + L::OFF_Q;
+  uint8_t* k_s = smem + L::OFF_K;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_CTRL);
+  uint64_t* full_k = bars;
+  uint64_t* empty_k = bars + S;
+  uint64_t* q_full = bars + 2 * S;
+  uint64_t* q_empty = bars + 2 * S + 1;
+  uint64_t* acc_full = bars + 2 * S + 2;                  // [RT][NACC]
+  uint64_t* acc_empty = bars + 2 * S + 2 + RT * NACC;     // [RT][NACC]
+  uint64_t* drain = bars + 2 * S + 2 + 2 * RT * NACC;     // [RT]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::NBARS);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  uint32_t* pk_done = tmem_slot + 2;                      // [8] units handed over by each filter warp
+  uint32_t* ep_done = tmem_slot + 10;                     // [8] units finished by the epilogue, per warp or job
+  int* row_n = reinterpret_cast<int*>(tmem_slot + 18);    // [RPU] kept counts (lists handed over in place)
+  uint8_t* list_mem = smem + L::OFF_LIST;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full_k[s], 1);
+      mbar_init(&empty_k[s], RT);
+    }
+    mbar_init(q_full, 1);
+    mbar_init(q_empty, RT);
+    for (int b = 0; b < RT * NACC; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], NQ);
+    }
+    for (int rt = 0; rt < RT; ++rt) mbar_init(&drain[rt], 1);
+    *abort_flag = 0;
+    for (int q = 0; q < 8; ++q) pk_done[q] = ep_done[q] = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) tmem_alloc(tmem_slot, L::TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  const int n_qt = (Lq + RU - 1) / RU;
+  // A unit is (b, h, query rows, key part): with parts > 1 (grids that would
+  // leave SMs idle, as decoding a few positions against a long cache does)
+  // each query tile's key tiles are split into `parts` ranges, each part keeps
+  // its own top k, and a merge kernel combines them.
+  auto decode = [&](int u_, int& bh, int& qt, int& part) {
+    part = u_ % parts;
+    const int u = u_ / parts;
+    if (causal) {  // heaviest query tiles first
+      qt = n_qt - 1 - u / BH;
+      bh = u % BH;
+    } else {  // consecutive units share a head, so its K/V stay in L2
+      bh = u / n_qt;
+      qt = u % n_qt;
+    }
+  };
+  // Eq. 2's masks as a valid key prefix per row: causal (queries are the
+  // last Lq positions: key j is valid for query i iff j <= i + Lk - Lq) and
+  // the batch's key count.  A unit streams at least one key tile, all of it
+  // masked if its rows have no key, so that every pipeline stage runs.
+  const int coff = Lk - Lq;
+  auto kv_end = [&](int bh) { return kv_len ? min(max(__ldg(kv_len + bh / H), 0), Lk) : Lk; };
+  auto key_tiles = [&](int bh, int i_end) {  // key tiles of the query rows below i_end
+    int kend = min(kv_end(bh), causal ? min(i_end + coff, Lk) : Lk);
+    kend = max(kend, 1);
+    return (kend + N - 1) / N;
+  };
+  auto row_limit = [&](int bh, int i) {  // keys j < limit are valid for query i
+    return static_cast<uint32_t>(min(kv_end(bh), causal ? min(i + 1 + coff, Lk) : Lk));
+  };
+  // key tiles [t0, t1) of a unit's part; a part left without tiles streams one
+  // fully masked tile (empty = true) so that every stage keeps its handshakes
+  auto tile_range = [&](int bh, int qt, int part, int& t0, int& t1, bool& empty) {
+    const int nk = key_tiles(bh, (qt + 1) * RU);
+    t0 = static_cast<int>(static_cast<long long>(part) * nk / parts);
+    t1 = static_cast<int>(static_cast<long long>(part + 1) * nk / parts);
+    empty = t1 <= t0;
+    if (empty) {
+      t0 = 0;
+      t1 = 1;
+    }
+  };
+
+  // The bound pass: the n_full key tiles that are valid for every row of the
+  // unit are scored twice, first only for their group maxima, so that the main
+  // pass starts with a threshold (RowList::bound_begin).  The second GEMM costs
+  // less than the candidates it saves: bounds over a quarter, three quarters and
+  // all of the keys took 20.3, 19.3 and 18.4 ms at L = 65536, k = 64.  Where the
+  // keys come from device memory each time it covers a quarter of them
+  // (bound_den = 4, see bound_divisor()).  Fewer than 6 k keys give no useful bound.
+  auto bound_tiles = [&](int bh, int qt, int t0, int t1, bool empty) {
+    if (empty) return 0;
+    const int nb = (min(t1, static_cast<int>(row_limit(bh, qt * RU)) / N) - t0) / bound_den;
+    return nb * N >= 6 * topk ? nb : 0;
+  };
+
+  // entry t of row r of filter warp `job`'s lists
+  auto list_at = [&](int job, int r, int t) {
+    const uint32_t base = smem_u32(list_mem + job * List::bytes(cap)) + List::M::kRecBytes;
+    return make_uint2(__float_as_uint(lds_f32(base + t * kScStep + r * 4)),
+                      lds_idx<IdxT>(base + cap * kScStep + t * kIxStep<IdxT> + r * static_cast<uint32_t>(sizeof(IdxT))));
+  };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    if (lane == 0) {
+      tma_prefetch_desc(&tmq);
+      tma_prefetch_desc(&tmk);
+    }
+    uint32_t it = 0, q_issued = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+      int bh, qt, part;
+      decode(u, bh, qt, part);
+      if (!warp_wait(q_empty, (q_issued & 1u) ^ 1u, ctl, abort_flag)) break;
+      if (lane == 0) {
+        mbar_arrive_expect_tx(q_full, RT * L::Q_BYTES);
+        for (int rt = 0; rt < RT; ++rt)
+          for (int r = 0; r < R; ++r)
+            tma_load_3d(q_s + rt * L::Q_BYTES + r * BM * 128, &tmq, q_full, r * 64, qt * RU + rt * BM, bh);
+      }
+      ++q_issued;
+      int t0, t1;
+      bool empty;
+      tile_range(bh, qt, part, t0, t1, empty);
+      const int nb = bound_tiles(bh, qt, t0, t1, empty);
+      for (int i = -nb; i < t1 - t0; ++i) {
+        const int kt = t0 + (i < 0 ? i + nb : i);
+        const int s = it % S;
+        const uint32_t ph = (it / S) & 1u;
+        if (!warp_wait(&empty_k[s], ph ^ 1u, ctl, abort_flag)) {
+          ok = false;
+          break;
+        }
+        if (lane == 0) {
+          if (ctl.debug_skip_arrive && it == 1) {
+            // testing hook: withhold this stage so the consumers' waits run out
+          } else {
+            mbar_arrive_expect_tx(&full_k[s], L::KST_BYTES);
+            for (int r = 0; r < R; ++r)
+              tma_load_3d(k_s + static_cast<size_t>(s) * L::KST_BYTES + r * N * 128, &tmk, &full_k[s], r * 64,
+                          kt * N, bh);
+          }
+        }
+        ++it;
+      }
+    }
+    // drain: every issued copy must have landed before the CTA may exit
+    if (lane == 0) {
+      for (uint32_t back = 1; back <= static_cast<uint32_t>(S) && back <= it; ++back) {
+        const uint32_t t = it - back;
+        if (ctl.debug_skip_arrive && t == 1) continue;
+        mbar_drain(&full_k[t % S], (t / S) & 1u, ctl);
+      }
+      if (q_issued > 0) mbar_drain(q_full, (q_issued - 1) & 1u, ctl);
+    }
+    __syncwarp();
+  } else if (warp <= RT) {
+    // ------------------------------------------------------------ MMA issuers
+    const int rt = warp - 1;
+    uint32_t it = 0, acc_it = 0, qi = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++qi) {
+      int bh, qt, part;
+      decode(u, bh, qt, part);
+      if (!warp_wait(q_full, qi & 1u, ctl, abort_flag)) break;
+      tc_fence_after();
+      int t0, t1;
+      bool empty;
+      tile_range(bh, qt, part, t0, t1, empty);
+      const int nb = bound_tiles(bh, qt, t0, t1, empty);
+      for (int i = -nb; i < t1 - t0; ++i, ++it, ++acc_it) {
+        const int s = it % S;
+        const int b = rt * NACC + acc_it % NACC;
+        if (!warp_wait(&full_k[s], (it / S) & 1u, ctl, abort_flag) ||
+            !warp_wait(&acc_empty[b], ((acc_it / NACC) & 1u) ^ 1u, ctl, abort_flag)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        if (lane == 0) {
+          const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(b * N);
+          const uint32_t qa = smem_u32(q_s) + rt * L::Q_BYTES;
+          const uint32_t ka = smem_u32(k_s + static_cast<size_t>(s) * L::KST_BYTES);
+#pragma unroll
+          for (int st = 0; st < D / 16; ++st) {
+            const uint32_t r = st / 4, off = (st % 4) * 32;
+            mma_bf16_ss(d_tmem, sdesc_k128(qa + r * BM * 128 + off), sdesc_k128(ka + r * N * 128 + off), IDESC,
+                        st > 0 ? 1u : 0u);
+          }
+          mma_commit(&empty_k[s]);
+          mma_commit(&acc_full[b]);
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      if (lane == 0) mma_commit(q_empty);
+      __syncwarp();
+    }
+    // drain: all issued MMAs must complete before TMEM is freed
+    if (lane == 0) {
+      mma_commit(&drain[rt]);
+      mbar_drain(&drain[rt], 0, ctl);
+    }
+    __syncwarp();
+  } else if (warp >= 4 && warp < 4 + 4 * RT) {
+    // ------------------------------------------------------------ filters
+    const int quad = warp & 3;       // TMEM lane quarter
+    const int rt = (warp - 4) >> 2;  // query tile
+    if (quad < NQ) {                 // lanes of the MMA tile that belong to the unit
+      const int job = rt * NQ + quad;
+      const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
+      uint32_t acc_it = 0;
+      List list;
+      list.bind(list_mem + job * List::bytes(cap), cap, topk);
+      bool ok = true;
+      uint32_t s = 0;  // units done
+      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++s) {
+        int bh, qt, part;
+        decode(u, bh, qt, part);
+        const int i0 = qt * RU + rt * BM + quad * 32;  // the warp's first query row
+        const int i_row = i0 + lane;
+        if (!L::kPark && parts == 1 && s > 0) {  // the lists handed over in place are free again
+          for (int h = 0; ok && h < L::NS; ++h)
+            ok = wait_count(&ep_done[job * L::NS + h], s, ctl, abort_flag);
+          if (!ok) break;
+        }
+        float tau0 = i_row < Lq ? -INFINITY : INFINITY;
+        int t0, t1;
+        bool empty;
+        tile_range(bh, qt, part, t0, t1, empty);
+        const uint32_t lim = empty ? 0u : row_limit(bh, i_row);
+        const int lim_min = empty ? 0 : static_cast<int>(row_limit(bh, i0));  // smallest limit of the warp's rows
+        const int nb = bound_tiles(bh, qt, t0, t1, empty);
+        if (nb > 0) {
+          // groups of 64 keys, or as many fewer as leave a group per class
+          int group = 64;
+          while (group > 4 && nb * N < group * classes) group >>= 1;
+          const int M = min(classes, (nb * N / group) & ~15);
+          list.bound_begin(M);
+          int slot = 0;  // M is a multiple of 16: a tile's slots do not wrap
+          auto stretch = [&](auto g) {
+            constexpr int G = decltype(g)::value;
+            for (int i = 0; i < nb; ++i, ++acc_it) {
+              const int b = rt * NACC + acc_it % NACC;
+              if (!warp_wait(&acc_full[b], (acc_it / NACC) & 1u, ctl, abort_flag)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              list.template bound_tile<N, G>(tmem_base + lane_base + static_cast<uint32_t>(b * N), slot);
+              tc_fence_before();
+              __syncwarp();
+              mbar_arrive_if(lane == 0, &acc_empty[b]);
+              slot = slot + N / G >= M ? 0 : slot + N / G;
+            }
+          };
+          if (group == 64)
+            stretch(std::integral_constant<int, 64>{});
+          else if (group == 32)
+            stretch(std::integral_constant<int, 32>{});
+          else if (group == 16)
+            stretch(std::integral_constant<int, 16>{});
+          else if (group == 8)
+            stretch(std::integral_constant<int, 8>{});
+          else
+            stretch(std::integral_constant<int, 4>{});
+          if (!ok) break;
+          const float t = list.bound_end(M);
+          if (i_row < Lq) tau0 = t;
+        }
+        list.begin(tau0);
+        for (int kt = t0; kt < t1; ++kt, ++acc_it) {
+          const int b = rt * NACC + acc_it % NACC;
+          if (!warp_wait(&acc_full[b], (acc_it / NACC) & 1u, ctl, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t taddr = tmem_base + lane_base + static_cast<uint32_t>(b * N);
+          const uint32_t jt = static_cast<uint32_t>(kt * N);
+          const bool masked = static_cast<int>(jt) + N > lim_min;  // some key is not valid for some row
+#pragma unroll 1
+          for (int c = 0; c < N; c += kOffer) {
+            float va[kOffer], ma[kOffer / 8];
+            load_chunk<kOffer / 8>(taddr + c, va, ma);
+            tmem_wait_tied(va, ma);
+            if (c + kOffer == N) {
+              tc_fence_before();
+              __syncwarp();
+              mbar_arrive_if(lane == 0, &acc_empty[b]);
+            }
+            if (masked) {  // a group's maximum is then taken over its valid keys
+#pragma unroll
+              for (int e = 0; e < kOffer; ++e)
+                if (jt + c + e >= lim) va[e] = -INFINITY;
+#pragma unroll
+              for (int g = 0; g < kOffer / 8; ++g)
+                ma[g] = max3f(max3f(va[8 * g], va[8 * g + 1], va[8 * g + 2]),
+                              max3f(va[8 * g + 3], va[8 * g + 4], va[8 * g + 5]), fmaxf(va[8 * g + 6], va[8 * g + 7]));
+            }
+            list.template offer<kOffer / 8>(va, ma, jt + c);
+          }
+        }
+        if (!ok) break;
+        list.finish(parts > 1 ? 0 : hand - topk);
+        const int list_n = list.count();
+        __syncwarp();  // the lists are read across lanes below
+        if (parts > 1) {  // this part's kept keys, for the merge
+          const size_t prow0 = (static_cast<size_t>(part) * BH + bh) * Lq + i0;
+          for (int r = 0; r < 32 && i0 + r < Lq; ++r) {
+            const int n = __shfl_sync(0xffffffffu, list_n, r);
+            for (int t = lane; t < n; t += 32) part_keys[(prow0 + r) * topk + t] = list_at(job, r, t);
+          }
+          if (i_row < Lq) part_n[prow0 + lane] = list_n;
+          __syncwarp();
+        } else if constexpr (L::kPark) {
+          // slot s % SL last held unit s - SL, whose epilogue must be done
+          if (s >= L::SL) {
+            for (int h = 0; ok && h < L::NS; ++h)
+              ok = wait_count(&ep_done[job * L::NS + h], s - L::SL + 1, ctl, abort_flag);
+            if (!ok) break;
+          }
+          const size_t slot = (static_cast<size_t>(blockIdx.x) * NJ + job) * L::SL + s % L::SL;
+          uint2* pk = park + slot * 32 * hand;
+          for (int r = 0; r < 32; ++r) {
+            const int n = __shfl_sync(0xffffffffu, list_n, r);
+            for (int t = lane; t < n; t += 32) pk[r * hand + t] = list_at(job, r, t);
+          }
+          park_n[slot * 32 + lane] = list_n;
+          __syncwarp();
+          st_release_u32(&pk_done[job], s + 1);
+        } else {
+          row_n[job * 32 + lane] = list_n;
+          __syncwarp();
+          st_release_u32(&pk_done[job], s + 1);
+        }
+      }
+    }
+  } else if (warp >= 4 && parts == 1) {
+    // ------------------------------------------------------------ epilogue
+    // Warp e takes RS rows of filter warp e / NS, then of filter warp
+    // (e + NE) / NS ..., unit by unit.
+    const int e = warp - (4 + 4 * RT);
+    uint2* buf = reinterpret_cast<uint2*>(list_mem + NJ * List::bytes(cap)) + e * topk;
+    uint32_t s = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++s) {
+      int bh, qt, part;
+      decode(u, bh, qt, part);
+      for (int w = e; w < NJ * L::NS; w += NE) {
+        const int job = w / L::NS, r0 = (w % L::NS) * L::RS;
+        if (!wait_count(&pk_done[job], s + 1, ctl, abort_flag)) {
+          ok = false;
+          break;
+        }
+        const int i0 = qt * RU + (job / NQ) * BM + (job % NQ) * 32 + r0;
+        const __nv_bfloat16* vb = v + static_cast<size_t>(bh) * Lk * D;
+        const size_t slot = (static_cast<size_t>(blockIdx.x) * NJ + job) * L::SL + s % L::SL;
+        int nv = 0;  // lane r: the kept count of row r
+        if (lane < L::RS) {
+          if constexpr (L::kPark)
+            nv = __ldcg(park_n + slot * 32 + r0 + lane);
+          else
+            nv = row_n[job * 32 + r0 + lane];
+        }
+        for (int r = 0; r < L::RS && i0 + r < Lq; ++r) {
+          const int n = __shfl_sync(0xffffffffu, nv, r);
+          const size_t orow = static_cast<size_t>(bh) * Lq + i0 + r;
+          int32_t* ir = idx ? idx + orow * topk : nullptr;
+          float* fr = score ? score + orow * topk : nullptr;
+          auto go = [&](auto&& load) {
+            // k + 32 candidates at most, rounded up to whole slots of 32
+            if constexpr (L::kPark) {
+              if (topk <= 32)
+                finish_row<__nv_bfloat16, D, 2, 1>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+              else if (topk <= 64)
+                finish_row<__nv_bfloat16, D, 3, 2>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+              else if (topk <= 128)
+                finish_row<__nv_bfloat16, D, 5, 4>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+              else if constexpr (RT == 1)
+                finish_row<__nv_bfloat16, D, 9, 8>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+            } else {
+              if (topk <= 256)
+                finish_row<__nv_bfloat16, D, 9, 8>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+              else
+                finish_row<__nv_bfloat16, D, 17, 16>(load, n, topk, buf, vb, out + orow * D, ir, fr);
+            }
+          };
+          if constexpr (L::kPark) {
+            const uint2* pk = park + (slot * 32 + r0 + r) * hand;
+            go([pk](int t) { return __ldcg(pk + t); });
+          } else {
+            go([&, r](int t) { return list_at(job, r0 + r, t); });
+          }
+        }
+        __syncwarp();
+        st_release_u32(&ep_done[w], s + 1);
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, L::TMEM_COLS);
+  }
+}
+
+// Key parts per query tile: split only grids that would leave at least half
+// the SMs idle (a few query tiles against many keys), into as many parts as
+// fill the SMs in one wave, each with at least 4 key tiles.
+int tc_parts(const AttnArgs& a, int num_sms, int N, int ru) {
+  const long long units = static_cast<long long>(a.B) * a.H * ((a.Lq + ru - 1) / ru);
+  if (units * 2 > num_sms) return 1;
+  const int kend_min = a.causal ? std::min(a.Lk, ru + (a.Lk - a.Lq)) : a.Lk;  // query tile 0's key range
+  const int nk_min = (kend_min + N - 1) / N;
+  long long p = num_sms / units;
+  p = std::min<long long>(p, nk_min / 4);
+  p = std::min<long long>(p, 8);
+  return static_cast<int>(std::max<long long>(p, 1));
+}
+
+size_t parts_bytes(const AttnArgs& a, int parts) {
+  if (parts <= 1) return 0;
+  const size_t rows = static_cast<size_t>(a.B) * a.H * a.Lq;
+  return static_cast<size_t>(parts) * rows * (static_cast<size_t>(a.topk) * 8 + 4);
+}
+
+// The share of the keys that the bound pass covers.  With one query tile per
+// head nobody else reads a head's keys; once they are several times what L2
+// holds (129 MB) a second pass over them reads device memory again.  Measured,
+// all of the keys against a quarter: 1.07 GB of keys (one position each,
+// d = 128) 589 and 433 us, 1.6 GB (128 positions) 1474 and 1312 us, but 0.40 GB
+// (128 positions, d = 64) 336 and 391 us.
+int bound_divisor(const AttnArgs& a) {
+  const double key_bytes = 2.0 * a.B * a.H * a.Lk * a.d;
+  return a.Lq <= BM && key_bytes > 512e6 ? 4 : 1;
+}
+
+constexpr int kMergeWarps = 8;
+
+// Merges a row's `parts` kept lists (each the exact top k of its key range, in
+// index order, so their union holds the row's top k), one warp per row.  The
+// k-th largest score of the union is found bit by bit on the ordered scores
+// (below the bits all of them share), the keys above it and the first ties at
+// it are compacted in place (part-major order is index order), and the row is
+// finished as in the single-pass kernel.
+template <int D, int KPL>
+__global__ void __launch_bounds__(kMergeWarps * 32)
+    attn_merge_kernel(const uint2* __restrict__ part_keys, const int* __restrict__ part_n, int parts, int BH, int Lq,
+                      int Lk, int topk, const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out,
+                      int32_t* __restrict__ idx, float* __restrict__ score) {
+  extern __shared__ uint2 mk_all[];  // [kMergeWarps][parts * topk]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint2* mk = mk_all + static_cast<size_t>(warp) * parts * topk;
+  const long long rows = static_cast<long long>(BH) * Lq;
+  for (long long r = static_cast<long long>(blockIdx.x) * kMergeWarps + warp; r < rows;
+       r += static_cast<long long>(gridDim.x) * kMergeWarps) {
+    int P = 0;
+    uint32_t hi = 0u, lo = 0xffffffffu;
+    for (int p = 0; p < parts; ++p) {
+      const long long pr = static_cast<long long>(p) * rows + r;
+      // counts and keys are checked before use: after a kernel that stopped
+      // early (a wait ran out) they may never have been written
+      const int n = min(max(__ldg(part_n + pr), 0), topk);
+      for (int t0 = 0; t0 < n; t0 += 32) {
+        const int t = t0 + lane;
+        uint2 e = make_uint2(0u, 0u);
+        bool live = t < n;
+        if (live) {
+          e = __ldg(part_keys + pr * topk + t);
+          live = e.y < static_cast<uint32_t>(Lk);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, live);
+        if (live) {
+          const uint32_t o = ord_f32(__uint_as_float(e.x));
+          mk[P + __popc(bal & ((1u << lane) - 1u))] = make_uint2(o, e.y);
+          hi = max(hi, o);
+          lo = min(lo, o);
+        }
+        P += __popc(bal);
+      }
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    __syncwarp();
+    int n = P;
+    if (P > topk) {
+      uint32_t thr = hi;
+      int c_thr = 0;  // entries >= thr, once a probe has counted them
+      if (lo != hi) {
+        const int top = 31 - __clz(lo ^ hi);
+        thr = top == 31 ? 0u : hi & ~((2u << top) - 1u);
+        c_thr = P;
+        for (int b = top; b >= 0 && c_thr != topk; --b) {
+          const uint32_t cand = thr | (1u << b);
+          int c = 0;
+          for (int i = lane; i < P; i += 32) c += mk[i].x >= cand ? 1 : 0;
+          c = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(c)));
+          if (c >= topk) {
+            thr = cand;
+            c_thr = c;
+          }
+        }
+      }
+      // keep what is above thr and, where more than k entries reach it, the
+      // first of those equal to it
+      int above = 0;
+      for (int i = lane; i < P; i += 32) above += mk[i].x > thr ? 1 : 0;
+      above = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(above)));
+      int eq_left = c_thr == topk ? P : topk - above;
+      int w = 0;
+      for (int i0 = 0; i0 < P; i0 += 32) {
+        const int i = i0 + lane;
+        const uint2 e = i < P ? mk[i] : make_uint2(0u, 0u);
+        const bool eq = i < P && (c_thr == topk ? e.x >= thr : e.x == thr);
+        const unsigned beq = __ballot_sync(0xffffffffu, eq);
+        const unsigned below = (1u << lane) - 1u;
+        const bool take = (i < P && e.x > thr) || (eq && __popc(beq & below) < eq_left);
+        const unsigned bt = __ballot_sync(0xffffffffu, take);
+        eq_left -= __popc(beq);
+        if (take) mk[w + __popc(bt & below)] = e;
+        w += __popc(bt);
+        __syncwarp();
+      }
+      n = min(w, topk);
+    }
+    const int bh = static_cast<int>(r / Lq);
+    finish_kept<__nv_bfloat16, D, KPL>(
+        [mk](int t) { return make_uint2(__float_as_uint(unord_f32(mk[t].x)), mk[t].y); }, n, topk,
+        v + static_cast<size_t>(bh) * Lk * D, out + r * D, idx ? idx + r * topk : nullptr,
+        score ? score + r * topk : nullptr);
+    __syncwarp();
+  }
+}
+
+template <int D, int KPL>
+int launch_merge(const AttnArgs& a, const uint2* part_keys, const int* part_n, int parts, int num_sms,
+                 cudaStream_t st) {
+  const size_t msmem = static_cast<size_t>(kMergeWarps) * parts * a.topk * sizeof(uint2);
+  auto merge = attn_merge_kernel<D, KPL>;
+  if (msmem > 48 * 1024 &&
+      cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(msmem)) != cudaSuccess)
+    return -1;
+  const long long rows = static_cast<long long>(a.B) * a.H * a.Lq;
+  long long mgrid = (rows + kMergeWarps - 1) / kMergeWarps;
+  if (mgrid > 16LL * num_sms) mgrid = 16LL * num_sms;
+  merge<<<static_cast<unsigned>(mgrid), kMergeWarps * 32, msmem, st>>>(
+      part_keys, part_n, parts, a.B * a.H, a.Lq, a.Lk, a.topk, static_cast<const __nv_bfloat16*>(a.v),
+      static_cast<__nv_bfloat16*>(a.out), a.idx, a.score);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// What a kernel variant needs for a call.
+struct TcPlan {
+  int ru = 0, N = 0, parts = 1, n_units = 0, grid = 0;
+  size_t park = 0, bytes = 0;
+  bool fits = false;
+};
+
+template <int D, typename IdxT, int RT, int RPU>
+struct Variant {
+  using L = Layout<D, IdxT, RT, RPU>;
+
+  static TcPlan plan(const AttnArgs& a, int num_sms) {
+    TcPlan p;
+    p.ru = RT * RPU;
+    p.N = L::N;
+    p.fits = L::fits(a.topk);
+    p.parts = RT == 1 ? tc_parts(a, num_sms, L::N, RPU) : 1;
+    p.n_units = a.B * a.H * ((a.Lq + p.ru - 1) / p.ru) * p.parts;
+    p.grid = p.n_units < num_sms ? p.n_units : num_sms;
+    p.park = p.parts == 1 ? L::park_bytes(p.grid, a.topk) : 0;
+    p.bytes = p.park + parts_bytes(a, p.parts);
+    return p;
+  }
+
+  static int launch(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st) {
+    const int BH = a.B * a.H;
+    const TcPlan p = plan(a, num_sms);
+    CUtensorMap tmq, tmk;
+    if (!make_tmap_bf16_3d(&tmq, a.q, D, a.Lq, BH, BM)) return -1;
+    if (!make_tmap_bf16_3d(&tmk, a.k, D, a.Lk, BH, L::N)) return -1;
+    // At least 120 KB so that a second CTA never shares the SM: each CTA takes
+    // all TMEM columns it needs for its whole (persistent) lifetime.
+    const size_t smem = std::max<size_t>(L::bytes(a.topk), 120 * 1024);
+    auto kern = attn_tc_kernel<D, IdxT, RT, RPU>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
+        cudaSuccess)
+      return -1;
+    if (p.bytes && (!a.workspace || a.workspace_bytes < p.bytes)) return -1;
+    uint8_t* ws = static_cast<uint8_t*>(a.workspace);
+    uint2* park = nullptr;
+    int* park_n = nullptr;
+    if (p.park) {
+      park = reinterpret_cast<uint2*>(ws);
+      park_n = reinterpret_cast<int*>(park + static_cast<size_t>(p.grid) * L::park_keys_per_cta(a.topk));
+    }
+    uint2* part_keys = nullptr;
+    int* part_n = nullptr;
+    if (p.parts > 1) {
+      const size_t rows = static_cast<size_t>(BH) * a.Lq;
+      part_keys = reinterpret_cast<uint2*>(ws + p.park);
+      part_n = reinterpret_cast<int*>(part_keys + static_cast<size_t>(p.parts) * rows * a.topk);
+      // counts start at 0, so that rows a stopped kernel never reached merge as empty
+      if (cudaMemsetAsync(part_n, 0, static_cast<size_t>(p.parts) * rows * sizeof(int), st) != cudaSuccess) return -1;
+    }
+    kern<<<p.grid, kThreads, smem, st>>>(tmq, tmk, static_cast<const __nv_bfloat16*>(a.v),
+                                         static_cast<__nv_bfloat16*>(a.out), BH, a.H, a.Lq, a.Lk, a.topk,
+                                         L::cap(a.topk), L::classes(a.topk), bound_divisor(a), a.causal, a.kv_len, p.n_units, p.parts, part_keys, part_n,
+                                         a.idx, a.score, park, park_n, ctl);
+    if (cudaGetLastError() != cudaSuccess) return -1;
+    if (p.parts == 1) return 1;
+    int rc;
+    if (a.topk <= 64)
+      rc = launch_merge<D, 2>(a, part_keys, part_n, p.parts, num_sms, st);
+    else if (a.topk <= 128)
+      rc = launch_merge<D, 4>(a, part_keys, part_n, p.parts, num_sms, st);
+    else if (a.topk <= 256)
+      rc = launch_merge<D, 8>(a, part_keys, part_n, p.parts, num_sms, st);
+    else
+      rc = launch_merge<D, 16>(a, part_keys, part_n, p.parts, num_sms, st);
+    return rc == 0 ? 2 : -1;
+  }
+};
+
+// Which variant serves a call: f is called with the Variant.
+// - Two query tiles per unit share each key tile and give an SM eight filter
+//   warps, which is faster for long rows (L = 65536, k = 64: 18.4 ms against
+//   31.8; L = 16384: 2.3 against 2.9), but they leave the epilogue half the
+//   warps and the rows half the memory: it is used where the lists fit (k up to
+//   68 at d = 64), the grid fills the SMs, rows have 128 k keys on average and no
+//   selection is asked for (causal L = 8192, k = 64: 0.75 ms against 0.68).
+// - Else one query tile; and, for k beyond what 128 rows' lists can hold, units
+//   of 64 or 32 query rows.
+// Indices take 16 bits up to 65,536 keys.
+template <int D, typename IdxT, typename F>
+auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
+  if constexpr (D == 64 && sizeof(IdxT) == 2) {
+    const long long units2 = static_cast<long long>(a.B) * a.H * ((a.Lq + 2 * BM - 1) / (2 * BM));
+    const int keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk;
+    if (Layout<D, IdxT, 2, BM>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
+      return f(Variant<D, IdxT, 2, BM>{});
+  }
+  if (Layout<D, IdxT, 1, BM>::fits(a.topk)) return f(Variant<D, IdxT, 1, BM>{});
+  if (Layout<D, IdxT, 1, 64>::fits(a.topk)) return f(Variant<D, IdxT, 1, 64>{});
+  return f(Variant<D, IdxT, 1, 32>{});
+}
+
+// The two calls of attn_tc.cu for one head size.
+template <int D>
+size_t tc_bytes(const AttnArgs& a, int num_sms) {
+  auto f = [&](auto v) { return decltype(v)::plan(a, num_sms).bytes; };
+  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+}
+
+template <int D>
+int tc_launch(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st) {
+  auto f = [&](auto v) { return decltype(v)::launch(a, ctl, num_sms, st); };
+  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+}
+
+}  // namespace
+
+}  // namespace topk

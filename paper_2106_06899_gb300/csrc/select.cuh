@@ -20,26 +20,9 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "rowlist.cuh"
 
 namespace topk {
-
-__device__ __forceinline__ uint32_t ord_f32(float s) {
-  const uint32_t u = __float_as_uint(s + 0.0f);  // -0 -> +0
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ float unord_f32(uint32_t o) {
-  const uint32_t u = (o & 0x80000000u) ? (o & 0x7FFFFFFFu) : ~o;
-  return __uint_as_float(u);
-}
-
-__device__ __forceinline__ uint64_t make_key(float s, uint32_t j) {
-  return (static_cast<uint64_t>(ord_f32(s)) << 32) | static_cast<uint64_t>(~j);
-}
-
-__device__ __forceinline__ float key_score(uint64_t key) { return unord_f32(static_cast<uint32_t>(key >> 32)); }
-
-__device__ __forceinline__ uint32_t key_index(uint64_t key) { return ~static_cast<uint32_t>(key); }
 
 // The heap of one row: a min-heap of its k best packed keys in shared memory
 // ([slot][row] layout, ROWS rows per slot).  push() offers one key; sort()
