@@ -158,7 +158,7 @@ int run_attn(const AttnArgs& a, cudaStream_t st) {
   b.workspace_bytes = ws;
   int n = attn_tc(b, ctl, dev->num_sms, st);
   if (buf) cudaFreeAsync(buf, st);
-  if (n == 0) n = attn_simt(a, st);
+  if (n == 0) n = attn_simt(a, dev->num_sms, st);
   if (n == 0) return TOPK_ERR_UNSUPPORTED;
   if (n < 0) return TOPK_ERR_CUDA;
   t_last_launches = n;

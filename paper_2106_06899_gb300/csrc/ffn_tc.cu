@@ -36,7 +36,7 @@
 #include <algorithm>
 
 #include "kernels.h"
-#include "select.cuh"
+#include "rowlist.cuh"
 
 namespace topk {
 

@@ -10,9 +10,6 @@
 
 namespace topk {
 
-// topk above this uses 32-row CTAs on the SIMT path (heap memory is
-// topk x rows x 8 bytes of shared memory).
-constexpr int kSimtSmallRowsMaxK = 128;
 constexpr int kSimtMaxK = 512;
 // tcgen05 attention path limit: 128 rows' heaps up to k = 137, units of 64 or
 // 32 query rows up to 256 or 512 (heaps in shared memory)
@@ -54,7 +51,7 @@ struct FfnArgs {
 
 // Each launcher returns the number of kernel launches (> 0) on success,
 // 0 if it does not serve the given shape, -1 on a CUDA error.
-int attn_simt(const AttnArgs& a, cudaStream_t st);
+int attn_simt(const AttnArgs& a, int num_sms, cudaStream_t st);
 int attn_tc(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st);
 bool attn_tc_supports(const AttnArgs& a);
 // Bytes of device scratch attn_tc needs for these arguments on a device with

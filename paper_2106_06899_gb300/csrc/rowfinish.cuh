@@ -180,10 +180,12 @@ __device__ __forceinline__ void softmax_gather(const float (&s)[KPL], const uint
 
 // The exact top k (a row of m <= 32 KH candidates, entry 32 c + lane in slot c,
 // in index order) moved in order into buf (k entries of shared memory); returns
-// how many there are.  The k-th score is found bit by bit on the ordered scores,
+// how many there are, and in `low` a score that at least k entries reach (-inf
+// unless m > k).  The k-th score is found bit by bit on the ordered scores,
 // below the bits that all candidates share; ties at it go to the lower entries.
 template <int KH>
-__device__ __forceinline__ int select_into(const float (&s)[KH], const uint32_t (&j)[KH], int m, int k, uint2* buf) {
+__device__ __forceinline__ int select_into(const float (&s)[KH], const uint32_t (&j)[KH], int m, int k, uint2* buf,
+                                           float& low) {
   const int lane = threadIdx.x & 31;
   uint32_t o[KH];
   uint32_t hi = 0u, lo = 0xffffffffu;
@@ -224,6 +226,7 @@ __device__ __forceinline__ int select_into(const float (&s)[KH], const uint32_t 
       eq_left = k - static_cast<int>(__reduce_add_sync(0xffffffffu, n));
     }
   }
+  low = m > k ? unord_f32(thr) : -INFINITY;
   const uint32_t below = (1u << lane) - 1u;
   int w = 0;
 #pragma unroll
@@ -292,7 +295,9 @@ __device__ __forceinline__ void finish_row(Load&& load, int m, int topk, uint2* 
       s[c] = __uint_as_float(e.x);
       j[c] = e.y;
     }
-    n = select_into<KH>(s, j, m, topk, buf);
+    float low;
+    __syncwarp();  // buf may be where the candidates were read from
+    n = select_into<KH>(s, j, m, topk, buf, low);
   }
   finish_kept<T, D, KPL>([buf](int t) { return buf[t]; }, n, topk, vb, orow, idx_row, score_row);
   __syncwarp();  // buf is free again

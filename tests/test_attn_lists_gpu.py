@@ -97,3 +97,22 @@ def test_scores_of_infinity_and_nan_keys():
     T.topk_check()
     assert torch.isfinite(out).all() and torch.isfinite(score).all()
     assert not torch.isin(idx.cpu(), torch.tensor([0, 5, 700], dtype=torch.int32)).any()
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 16), ("f32", 64), ("f32", 128), ("bf16", 128)])
+@pytest.mark.parametrize("topk,Lk", [(1, 63), (64, 65), (128, 193), (129, 257), (128, 1000), (512, 700)])
+@pytest.mark.parametrize("rows", ["few", "many"])
+def test_cuda_core_lists(dtype, d, topk, Lk, rows):
+    # lists that are cut never, once or often; one or four rows per warp; bf16 runs here under a bit mask
+    B, H, Lq = (1, 1, 37) if rows == "few" else (7, 10, 140)
+    q, k, v = W.attention_inputs(B, H, Lq, Lk, d, dtype=dtype, seed=790 + topk + d)
+    mask = None
+    if dtype == "bf16":
+        mask = np.random.default_rng(topk).random((1, 1, Lq, Lk)) < 0.8
+    out, idx, score = T.attention(q.cuda(), k.cuda(), v.cuda(), topk, return_indices=True,
+                                  mask=None if mask is None else torch.from_numpy(mask).cuda())
+    T.topk_check()
+    sel = W.sample_rows(B * H * Lq, 300, seed=topk).numpy()
+    check_rows(q=q, k=k, v=v, rows=sel, gpu_out=out.float().cpu().reshape(-1, d).numpy()[sel],
+               gpu_idx=idx.cpu().reshape(-1, topk).numpy()[sel], gpu_score=score.cpu().reshape(-1, topk).numpy()[sel],
+               topk=topk, dtype=dtype, mask=mask)
