@@ -171,24 +171,6 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, const
   }
 }
 
-// Keeps the wait for a tcgen05.ld ahead of every use of what it loaded.
-template <int NV, int NM>
-__device__ __forceinline__ void tmem_wait_tied(float (&v)[NV], float (&m)[NM]) {
-  tmem_wait_ld();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) asm volatile("" : "+f"(v[i]));
-#pragma unroll
-  for (int i = 0; i < NM; ++i) asm volatile("" : "+f"(m[i]));
-}
-
-// 8 G consecutive TMEM columns of this thread's lane and the maxima of their
-// groups of eight.
-template <int G>
-__device__ __forceinline__ void load_chunk(uint32_t taddr, float (&v)[8 * G], float (&m)[G]) {
-#pragma unroll
-  for (int g = 0; g < G; ++g) tmem_ld8_max(taddr + 8 * g, reinterpret_cast<float(&)[8]>(v[8 * g]), m[g]);
-}
-
 template <int D, typename IdxT, int RT, int RPU>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,

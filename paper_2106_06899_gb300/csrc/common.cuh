@@ -324,6 +324,7 @@ __device__ __forceinline__ float tmem_ld_max<4>(uint32_t taddr) {
   asm volatile("tcgen05.ld.red.sync.aligned.32x32b.x4.max.f32 {%0, %1, %2, %3}, %4, [%5];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=f"(m)
                : "r"(taddr));
+  (void)r[0];
   return m;
 }
 template <>
@@ -334,6 +335,7 @@ __device__ __forceinline__ float tmem_ld_max<8>(uint32_t taddr) {
       "tcgen05.ld.red.sync.aligned.32x32b.x8.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, %8, [%9];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=f"(m)
       : "r"(taddr));
+  (void)r[0];
   return m;
 }
 template <>
@@ -346,6 +348,7 @@ __device__ __forceinline__ float tmem_ld_max<16>(uint32_t taddr) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=f"(m)
       : "r"(taddr));
+  (void)r[0];
   return m;
 }
 template <>
@@ -362,6 +365,7 @@ __device__ __forceinline__ float tmem_ld_max<32>(uint32_t taddr) {
         "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=f"(m)
       : "r"(taddr));
+  (void)r[0];
   return m;
 }
 template <>
@@ -383,10 +387,29 @@ __device__ __forceinline__ float tmem_ld_max<64>(uint32_t taddr) {
         "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]),
         "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63]), "=f"(m)
       : "r"(taddr));
+  (void)r[0];
   return m;
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// Keeps the wait for a tcgen05.ld ahead of every use of what it loaded.
+template <int NV, int NM>
+__device__ __forceinline__ void tmem_wait_tied(float (&v)[NV], float (&m)[NM]) {
+  tmem_wait_ld();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) asm volatile("" : "+f"(v[i]));
+#pragma unroll
+  for (int i = 0; i < NM; ++i) asm volatile("" : "+f"(m[i]));
+}
+
+// 8 G consecutive TMEM columns of this thread's lane and the maxima of their
+// groups of eight.
+template <int G>
+__device__ __forceinline__ void load_chunk(uint32_t taddr, float (&v)[8 * G], float (&m)[G]) {
+#pragma unroll
+  for (int g = 0; g < G; ++g) tmem_ld8_max(taddr + 8 * g, reinterpret_cast<float(&)[8]>(v[8 * g]), m[g]);
+}
 
 // ---------------------------------------------------------------- misc
 // Three-input maximum (one instruction on sm_100+); NaN inputs are ignored

@@ -37,6 +37,7 @@
 
 #include "kernels.h"
 #include "rowlist.cuh"
+#include "topk_attention.h"
 
 namespace topk {
 
@@ -51,14 +52,13 @@ constexpr int NBINS = 64;
 constexpr uint32_t A_BYTES = BM * KC * 2;  // 16 KB
 constexpr uint32_t B_BYTES = NT * KC * 2;  // 32 KB
 constexpr uint32_t ST_BYTES = A_BYTES + B_BYTES;
-constexpr int GR = 10;    // pending score groups per row (a 64-score call adds up to 8)
 constexpr size_t OFF_HIST = static_cast<size_t>(S) * ST_BYTES;
-constexpr size_t OFF_REC = OFF_HIST + static_cast<size_t>(NBINS) * BM * 4;
-constexpr size_t OFF_CTRL = OFF_REC + static_cast<size_t>(GR) * BM * 36;
+constexpr size_t OFF_STAGE = OFF_HIST + static_cast<size_t>(NBINS) * BM * 4;  // 32 scores per row
+constexpr size_t OFF_CTRL = OFF_STAGE + static_cast<size_t>(BM) * 32 * 4;
 constexpr size_t SMEM_A = 1024 + OFF_CTRL + 256;
 
 constexpr int kFinalThreads = 256;
-constexpr int kFinalMaxCand = 8192;  // candidates at or above the final bound held in shared memory
+constexpr int kFinalMaxCand = 4096;  // candidates at or above the final bound held in shared memory (32 KB: six CTAs per SM)
 constexpr int kFinalVec = 4;         // 16-byte candidate vectors each finalize thread loads per step
 
 struct Plan {
@@ -66,8 +66,7 @@ struct Plan {
   size_t off_cnt, off_tau, off_part, off_kept, bytes;
 };
 
-Plan make_plan(int N, int d_model, int d_ff, int topk, int num_sms) {
-  (void)d_model;
+Plan make_plan(int N, int d_ff, int topk, int num_sms, double slice_charge) {
   Plan p{};
   p.n_rt = (N + BM - 1) / BM;
   p.tiles = (d_ff + NT - 1) / NT;
@@ -83,7 +82,7 @@ Plan make_plan(int N, int d_model, int d_ff, int topk, int num_sms) {
     const long units = static_cast<long>(p.n_rt) * sl;
     const long waves = (units + num_sms - 1) / num_sms;
     const long per = (p.tiles + sl - 1) / sl;
-    const double cost = static_cast<double>(waves * per) + 0.5 * sl;
+    const double cost = static_cast<double>(waves * per) + slice_charge * sl;
     if (cost < best - 1e-9) {
       best = cost;
       p.n_sl = sl;
@@ -102,6 +101,20 @@ Plan make_plan(int N, int d_model, int d_ff, int topk, int num_sms) {
   p.off_kept = (p.off_part + rows_sl * sizeof(uint32_t) + 15) & ~size_t(15);
   p.bytes = p.off_kept + static_cast<size_t>(N) * topk * sizeof(uint64_t);  // kept keys per token
   return p;
+}
+
+// A slice costs its first tile's append and its share of the finalize: a tenth
+// of a key tile's time (300 tokens x 3072 keys, k = 64: twelve slices of one tile,
+// 79 us, against four of three tiles).  More slices can take more scratch, though: a
+// finer plan that would not fit the no-allocation entry's fixed buffer gives way to
+// the coarser one with half a tile per slice, so that nothing it took is refused.
+constexpr size_t kFixedScratch = TOPK_FFN_NOALLOC_SCRATCH_BYTES;
+Plan make_plan(int N, int d_model, int d_ff, int topk, int num_sms) {
+  (void)d_model;
+  const Plan fine = make_plan(N, d_ff, topk, num_sms, 0.1);
+  if (fine.bytes <= kFixedScratch) return fine;
+  const Plan coarse = make_plan(N, d_ff, topk, num_sms, 0.5);
+  return coarse.bytes < fine.bytes ? coarse : fine;
 }
 
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
@@ -131,6 +144,8 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, const
 struct RowCand {
   uint2* list;        // this (row, slice)'s candidate list, ascending key index
   uint32_t* hist;     // &hist[bin 0][row], stride BM
+  uint32_t hist_s;    // its shared address
+  uint32_t stage;     // shared address of the warp's staging area
   int cap, cnt, k;
   bool hist_on;
   float base, width, inv_width;
@@ -145,29 +160,15 @@ struct RowCand {
     return f > 0.0f ? static_cast<int>(f) : 0;
   }
 
-  __device__ __forceinline__ void add(float s, uint32_t j) {
-    if (cnt < cap) list[cnt] = make_uint2(__float_as_uint(s), j);
-    ++cnt;
-    if (hist_on) {
-      hist[bin(s) * BM] += 1u;
-    } else {
-      mn = fminf(mn, s);
-      mx = fmaxf(mx, s);
-    }
-  }
-
   // Raise L from the histogram (called between key tiles).
   __device__ __forceinline__ void refresh() {
     if (!hist_on) {
       if (cnt < k) return;
       // at least k candidates so far, every one of them >= mn
       L = fmaxf(L, mn);
-      base = mn;
-      width = fmaxf((mx - mn) * (1.0f / 48.0f), fmaxf(fabsf(mx), 1e-20f) * 1e-6f);
-      inv_width = 1.0f / width;
+      set_bins();
       hist[0] = static_cast<uint32_t>(cnt - 1);
       hist[bin(mx) * BM] += 1u;
-      hist_on = true;
       return;
     }
     // scan from the top bin down, eight bins per step: the eight loads are
@@ -206,68 +207,94 @@ struct RowCand {
     }
   }
 
-  // Pending score groups ([slot][row] records: 8 scores and the first key).
-  float4* rlo;
-  float4* rhi;
-  uint32_t* rj;
-  int rc;
-
-  // A score qualifies for the list if it reaches the shared bound Lg and
-  // beats the slice's own bound Ls strictly (see L above).
-  __device__ __forceinline__ static bool keep(float s, float Lg, float Ls) { return s >= Lg && s > Ls; }
-
-  // Expand every lane's records into its candidate list, lanes in lockstep:
-  // per record slot each lane forms the mask of its qualifying elements,
-  // then the warp appends one element per lane per step.
-  __device__ __forceinline__ void flush(float Lg, float Ls, bool active) {
-    const int mxr = __reduce_max_sync(0xffffffffu, static_cast<unsigned>(active ? rc : 0));
-    for (int i = 0; i < mxr; ++i) {
-      unsigned msk = 0;
-      uint32_t j0 = 0;
-      if (active && i < rc) {
-        const float4 a = rlo[i * BM];
-        const float4 b = rhi[i * BM];
-        j0 = rj[i * BM];
-        msk = (keep(a.x, Lg, Ls) ? 1u : 0u) | (keep(a.y, Lg, Ls) ? 2u : 0u) | (keep(a.z, Lg, Ls) ? 4u : 0u) |
-              (keep(a.w, Lg, Ls) ? 8u : 0u) | (keep(b.x, Lg, Ls) ? 16u : 0u) | (keep(b.y, Lg, Ls) ? 32u : 0u) |
-              (keep(b.z, Lg, Ls) ? 64u : 0u) | (keep(b.w, Lg, Ls) ? 128u : 0u);
-      }
-      while (__any_sync(0xffffffffu, msk != 0)) {
-        if (msk) {
-          const int e = __ffs(msk) - 1;
-          msk &= msk - 1;
-          const float v = e < 4 ? reinterpret_cast<const float*>(rlo + i * BM)[e]
-                                : reinterpret_cast<const float*>(rhi + i * BM)[e - 4];
-          add(v, j0 + e);
-        }
-      }
-    }
-    rc = 0;
-  }
-
-  // Offer 64 scores (key indices j0..j0+63): each group of 8 whose maximum
-  // qualifies (keep()) becomes one record (NaN, used for keys past d_ff,
-  // never does).
-  __device__ __forceinline__ void offer64(const float (&v)[64], uint32_t j0, float Lg, float Ls, bool active) {
-    float m[8];
+  // Offer 32 scores (key indices j0 .. j0 + 31, m[g] the maximum of their g-th
+  // eight): a score qualifies if it reaches the shared bound and beats the
+  // slice's own bound strictly (see L above), which is one compare with T.  The
+  // list has room (see the caller).  FIRST: some lane of the warp has no
+  // histogram yet and tracks its candidates' spread.
+  //
+  // The scores go to the warp's staging area in shared memory ([score / 4][row]
+  // vectors), each lane forms the mask of its qualifying ones, and the warp walks
+  // the masks in lockstep, one append and one histogram count per lane and step:
+  // as many steps as the row with most qualifying scores has.  Predicated stores
+  // for every score, without the walk, take two memory instructions per score
+  // whether it qualifies or not (18,000 cycles per 256-key tile; this: 9,000).
+  // While every row keeps everything (the first k keys), the staged scores are
+  // written row by row instead, 256 contiguous bytes each.
+  template <bool FIRST>
+  __device__ __forceinline__ void offer32(const float (&v)[32], const float (&m)[4], uint32_t j0, float T,
+                                          const uint2* warp_list, size_t row_stride) {
+    if (!__any_sync(0xffffffffu, max3f(fmaxf(m[0], m[1]), m[2], m[3]) > T)) return;
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t mask = 0;  // score e in bit 31 - e: the next one is a count of leading zeros
+#pragma unroll
+    for (int e = 0; e < 32; ++e) mask |= v[e] > T ? 0x80000000u >> e : 0u;
+    __syncwarp();
 #pragma unroll
     for (int g = 0; g < 8; ++g)
-      m[g] = max3f(max3f(v[8 * g], v[8 * g + 1], v[8 * g + 2]), max3f(v[8 * g + 3], v[8 * g + 4], v[8 * g + 5]),
-                   fmaxf(v[8 * g + 6], v[8 * g + 7]));
-    if (active) {
-      int r = rc;
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + g * 512 + lane * 16), "f"(v[4 * g]),
+                   "f"(v[4 * g + 1]), "f"(v[4 * g + 2]), "f"(v[4 * g + 3])
+                   : "memory");
+    if (FIRST && __all_sync(0xffffffffu, mask == 0xffffffffu && !hist_on)) {
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        if (keep(m[g], Lg, Ls)) {
-          rlo[r * BM] = make_float4(v[8 * g], v[8 * g + 1], v[8 * g + 2], v[8 * g + 3]);
-          rhi[r * BM] = make_float4(v[8 * g + 4], v[8 * g + 5], v[8 * g + 6], v[8 * g + 7]);
-          rj[r * BM] = j0 + 8 * g;
-          ++r;
+      for (int e = 0; e < 32; ++e) {
+        mn = fminf(mn, v[e]);
+        mx = fmaxf(mx, v[e]);
+      }
+      __syncwarp();
+#pragma unroll 4
+      for (int r = 0; r < 32; ++r) {
+        const int c = __shfl_sync(0xffffffffu, cnt, r);
+        const float x = lds_f32(stage + (lane >> 2) * 512 + r * 16 + (lane & 3) * 4);
+        const_cast<uint2*>(warp_list)[r * row_stride + c + lane] = make_uint2(__float_as_uint(x), j0 + lane);
+      }
+      cnt += 32;
+      return;
+    }
+    while (__any_sync(0xffffffffu, mask != 0u)) {
+      constexpr int U = 2;  // scores per lane and round: their loads overlap
+      bool act[U];
+      int e[U];
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        act[u] = mask != 0u;
+        e[u] = __clz(mask) & 31;
+        mask &= ~(0x80000000u >> e[u]);
+        x[u] = lds_f32(stage + (e[u] >> 2) * 512 + lane * 16 + (e[u] & 3) * 4);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.global.v2.b32 [%1], {%2, %3};\n\t}" ::"r"(
+                         static_cast<int>(act[u])),
+                     "l"(list + cnt), "r"(__float_as_uint(x[u])), "r"(j0 + e[u])
+                     : "memory");
+        count(act[u] && (!FIRST || hist_on), x[u]);
+        cnt += act[u] ? 1 : 0;
+        if (FIRST) {
+          mn = act[u] ? fminf(mn, x[u]) : mn;
+          mx = act[u] ? fmaxf(mx, x[u]) : mx;
         }
       }
-      rc = r;
     }
-    if (__any_sync(0xffffffffu, active && rc > GR - 8)) flush(Lg, Ls, active);
+  }
+
+  // One more candidate of score s in the histogram, if p.
+  __device__ __forceinline__ void count(bool p, float s) const {
+    const float f = fminf((s - base) * inv_width, static_cast<float>(NBINS - 1));
+    const uint32_t b = __float2uint_rz(f);  // below 0: 0
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q red.shared.add.u32 [%1], 1;\n\t}" ::"r"(
+                     static_cast<int>(p)),
+                 "r"(hist_s + b * (BM * 4))
+                 : "memory");
+  }
+
+  // The histogram's bins from the spread of the candidates so far.
+  __device__ __forceinline__ void set_bins() {
+    base = mn;
+    width = fmaxf((mx - mn) * (1.0f / 48.0f), fmaxf(fabsf(mx), 1e-20f) * 1e-6f);
+    inv_width = 1.0f / width;
+    hist_on = true;
   }
 
   // The list's exact top k by the total order (score descending, index
@@ -455,10 +482,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     rc.hist = hist_mem + row;
     rc.k = topk;
     rc.cap = cap;
-    rc.rlo = reinterpret_cast<float4*>(smem + OFF_REC) + row;
-    rc.rhi = reinterpret_cast<float4*>(smem + OFF_REC + static_cast<size_t>(GR) * BM * 16) + row;
-    rc.rj = reinterpret_cast<uint32_t*>(smem + OFF_REC + static_cast<size_t>(GR) * BM * 32) + row;
-    rc.rc = 0;
+    rc.hist_s = smem_u32(rc.hist);
+    rc.stage = smem_u32(smem + OFF_STAGE) + quad * 4096;
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
       int rt, sl, t0, t1;
       decode(u, rt, sl);
@@ -467,6 +492,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool row_ok = grow < N;
       const size_t rs = static_cast<size_t>(row_ok ? grow : 0) * n_sl + sl;
       rc.list = cand + rs * cap;
+      const uint2* warp_list = cand + (static_cast<size_t>(rt * BM + quad * 32) * n_sl + sl) * cap;  // the warp's first row
+      const size_t row_stride = static_cast<size_t>(n_sl) * cap;
       rc.cnt = 0;
       rc.hist_on = false;
       rc.base = 0.0f;
@@ -492,27 +519,57 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc_fence_after();
         const uint32_t taddr = tmem_base + lane_base + static_cast<uint32_t>(b * NT);
+        // a token past the last one keeps nothing
+        uint32_t below = ord_f32(Lg) - 1u;  // the largest score below Lg (below +0 comes -0, its equal)
+        if (below == 0x7fffffffu) --below;
+        const float T = row_ok ? fmaxf(Ls, shared_key ? unord_f32(below) : -INFINITY) : INFINITY;
+        const bool first = __any_sync(0xffffffffu, row_ok && !rc.hist_on);
 #pragma unroll 1
-        for (int c = 0; c < NT / 64; ++c) {
-          float v[64];
-          __syncwarp();
-          tmem_ld64(taddr + c * 64, v);
-          tmem_wait_ld();
-          if (c == NT / 64 - 1) {
+        for (int c = 0; c < NT / 32; ++c) {
+          float v[32], m[4];
+          load_chunk<4>(taddr + c * 32, v, m);
+          tmem_wait_tied(v, m);
+          if (c == NT / 32 - 1 && kt != t0) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[b]);
+            mbar_arrive_if(lane == 0, &acc_empty[b]);
           }
-          const uint32_t j0 = static_cast<uint32_t>(kt * NT + c * 64);
-          if (j0 + 64 > static_cast<uint32_t>(d_ff)) {
+          const uint32_t j0 = static_cast<uint32_t>(kt * NT + c * 32);
+          if (j0 + 32 > static_cast<uint32_t>(d_ff)) {  // keys past d_ff are never kept
 #pragma unroll
-            for (int e = 0; e < 64; ++e)
-              if (j0 + e >= static_cast<uint32_t>(d_ff)) v[e] = __uint_as_float(0x7fc00000u);  // NaN: never kept
+            for (int e = 0; e < 32; ++e)
+              if (j0 + e >= static_cast<uint32_t>(d_ff)) v[e] = -INFINITY;
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+              m[g] = max3f(max3f(v[8 * g], v[8 * g + 1], v[8 * g + 2]), max3f(v[8 * g + 3], v[8 * g + 4], v[8 * g + 5]),
+                           fmaxf(v[8 * g + 6], v[8 * g + 7]));
           }
-          rc.offer64(v, j0, Lg, Ls, row_ok);
+          if (first)
+            rc.offer32<true>(v, m, j0, T, warp_list, row_stride);
+          else
+            rc.offer32<false>(v, m, j0, T, warp_list, row_stride);
         }
-        // the tile's pending groups go to the list before the bound moves
-        if (__any_sync(0xffffffffu, row_ok && rc.rc > 0)) rc.flush(Lg, Ls, row_ok);
+        if (kt == t0) {
+          // The slice's first tile is read again for the histogram, whose bins its
+          // candidates' spread sets: the bounds then count every candidate from
+          // the first tile on (without it a slice appended two tiles whole and
+          // started counting after them).  Rows with fewer than kp candidates so
+          // far start counting later (refresh()).
+          const bool on = row_ok && rc.cnt >= rc.kp;
+          if (on) rc.set_bins();
+#pragma unroll 1
+          for (int c = 0; c < NT / 32; ++c) {
+            float v[32], m[4];
+            load_chunk<4>(taddr + c * 32, v, m);
+            tmem_wait_tied(v, m);
+            const int left = d_ff - (kt * NT + c * 32);  // keys of the chunk
+#pragma unroll
+            for (int e = 0; e < 32; ++e) rc.count(on && v[e] > T && e < left, v[e]);
+          }
+          tc_fence_before();
+          __syncwarp();
+          mbar_arrive_if(lane == 0, &acc_empty[b]);
+        }
         if (!row_ok) continue;
         rc.refresh();
         const uint32_t lkey = rc.L > -INFINITY ? ord_f32(rc.L) : 0u;
@@ -724,6 +781,63 @@ __global__ void __launch_bounds__(kFinalThreads)
     }
     __syncthreads();
   };
+  // Usually the row's bound leaves few enough candidates to collect them all at
+  // once and sort them in shared memory; the radix select below serves the rest.
+  for_each([&](bool valid, uint32_t o, uint32_t j) {
+    const int pa = warp_append(&n_keys, valid);
+    if (pa >= 0 && pa < kFinalMaxCand) keys[pa] = (static_cast<uint64_t>(o) << 32) | static_cast<uint64_t>(~j);
+  });
+  __syncthreads();
+  const int n_all = n_keys;
+  bool direct = n_all <= kFinalMaxCand;
+  if (n_all < topk) {  // fewer candidates than k: cannot happen unless the lists are inconsistent
+    if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
+    return;
+  }
+  if (direct) {
+    // keys[0 .. topk) become the kept keys, best first.  Sorting costs
+    // log^2 of the count: beyond the power of two that holds k, the k-th key is
+    // found first, bit by bit on the whole 64-bit keys (all are distinct), and
+    // only the k kept ones are sorted.
+    int p2 = 1;
+    while (p2 < topk) p2 <<= 1;
+    if (n_all > p2 && n_all <= kFinalMaxCand - topk) {
+      uint64_t thr = 0;
+      int c_thr = n_all;
+#pragma unroll 1
+      for (int b = 63; b >= 0 && c_thr != topk; --b) {
+        const uint64_t cd = thr | (1ull << b);
+        unsigned c = 0;
+        for (int i = tid; i < n_all; i += kFinalThreads) c += keys[i] >= cd ? 1u : 0u;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if ((tid & 31) == 0) csum[(b & 1) * 8 + (tid >> 5)] = c;
+        __syncthreads();  // two slots by turns: one barrier per bit
+        int all = 0;
+#pragma unroll
+        for (int w = 0; w < kFinalThreads / 32; ++w) all += static_cast<int>(csum[(b & 1) * 8 + w]);
+        if (all >= topk) {
+          thr = cd;
+          c_thr = all;
+        }
+      }
+      __syncthreads();
+      if (tid == 0) n_keys = 0;
+      __syncthreads();
+      uint64_t* kept_s = keys + kFinalMaxCand - topk;
+      for (int i0 = 0; i0 < n_all; i0 += kFinalThreads) {
+        const int i = i0 + tid;
+        const uint64_t key = i < n_all ? keys[i] : 0ull;
+        const int pa = warp_append(&n_keys, i < n_all && key >= thr);
+        if (pa >= 0 && pa < topk) kept_s[pa] = key;
+      }
+      __syncthreads();
+      for (int t = tid; t < topk; t += kFinalThreads) keys[t] = kept_s[t];
+      __syncthreads();
+      bitonic_desc(keys, topk);
+    } else {
+      bitonic_desc(keys, n_all);
+    }
+  }
   const int shifts[3] = {21, 10, 0};
   const uint32_t dmasks[3] = {0x7FFu, 0x7FFu, 0x3FFu};
   auto any = [](uint32_t, uint32_t) { return true; };
@@ -731,9 +845,12 @@ __global__ void __launch_bounds__(kFinalThreads)
   // radix select: the k-th largest ordered score among the candidates
   uint32_t prefix = 0, pmask = 0;
   int remaining = topk, n_eq = 0;
-  bool direct = false;
 #pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
+  for (int pass = 0; pass < 3 && !direct; ++pass) {
+    if (pass == 0) {
+      __syncthreads();
+      if (tid == 0) n_keys = 0;
+    }
     radix_digit(any, score_of, prefix, pmask, shifts[pass], dmasks[pass], remaining);
     const int digit = sh_digit, above = sh_above, count = sh_count;
     if (digit < 0) {  // fewer candidates than k: cannot happen unless the lists are inconsistent
