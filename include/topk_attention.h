@@ -275,10 +275,11 @@ int topk_ffn_fwd_noalloc(const void* x, const void* W1, const void* W2, void* ou
 
 /* Bytes of stream-ordered scratch the calls above take for these arguments
  * (0 if none).  Returns 0 as well when the arguments are invalid.
- *   - attention: the bf16 tensor-core kernel with split selection parks each
- *     work unit's kept keys for its epilogue warps: per CTA (one per SM, at
- *     most one per 128-query tile) 4 x 2 x topk x 32 keys of 8 bytes plus
- *     256 counts of 4 bytes, whatever Lq and Lk are.  Sized for the current
+ *   - attention: the bf16 tensor-core kernel hands each work unit's candidates
+ *     to its epilogue warps through it: per CTA (one per SM, at most one per
+ *     128-query tile) 16 x 32 rows of topk + 32 (rounded up to a multiple of
+ *     32) entries of 8 bytes plus a count of 4, whatever Lq and Lk are; none
+ *     where k is so large that the lists stay in shared memory.  Sized for the current
  *     device, or for 152 SMs (a GB300) when no device is visible.
  *   - feed-forward: linear in N (see topk_ffn_fwd). */
 size_t topk_attn_workspace_bytes(int B, int H, int Lq, int Lk, int d, int topk, int chunk, int dtype);

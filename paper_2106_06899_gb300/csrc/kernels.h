@@ -11,8 +11,7 @@
 namespace topk {
 
 constexpr int kSimtMaxK = 512;
-// tcgen05 attention path limit: 128 rows' heaps up to k = 137, units of 64 or
-// 32 query rows up to 256 or 512 (heaps in shared memory)
+// tcgen05 attention path limit: what the lists of a 32-row unit hold in shared memory
 constexpr int kTcMaxK = 512;
 
 struct AttnArgs {
@@ -23,7 +22,7 @@ struct AttnArgs {
   int B, H, Lq, Lk, d, topk, chunk, causal, dtype;
   int32_t* idx;
   float* score;
-  // device scratch of the tcgen05 split kernel (attn_tc_workspace_bytes)
+  // device scratch of the tcgen05 kernel (attn_tc_workspace_bytes)
   void* workspace = nullptr;
   size_t workspace_bytes = 0;
   // Eq. 2's masks besides causal: the key count of each batch ([B] int32,
@@ -55,8 +54,9 @@ int attn_simt(const AttnArgs& a, int num_sms, cudaStream_t st);
 int attn_tc(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st);
 bool attn_tc_supports(const AttnArgs& a);
 // Bytes of device scratch attn_tc needs for these arguments on a device with
-// num_sms SMs: the split kernel parks each unit's kept keys for its
-// epilogue warps (a fixed amount per CTA, nothing per query row); 0 otherwise.
+// num_sms SMs: the kernel hands each unit's candidates to its epilogue warps
+// through it (a fixed amount per CTA, nothing per query row), and key parts (small
+// grids) their kept lists to the merge; 0 otherwise.
 size_t attn_tc_workspace_bytes(const AttnArgs& a, int num_sms);
 
 size_t ffn_workspace_bytes(int N, int d_model, int d_ff, int topk);

@@ -18,9 +18,9 @@
 // dependent chain of about 150 instructions that the warp's lanes rarely share.
 // Here a bound taken from group maxima in a first pass over the keys (RowList)
 // leaves about 1.4 k candidates per row, each of them an append.  Measured,
-// heaps and lists: k = 64, L = 65,536, d = 64: 19.6 and 18.1 ms; k = 128,
+// heaps and lists: k = 64, L = 65,536, d = 64: 19.7 and 18.4 ms; k = 128,
 // L = 16,384 causal, d = 128: 15.8 and 8.9 ms; k = 256, L = 8,192: 11.3 and
-// 3.0 ms; k = 64, L = 512: 250 and 176 us.  What bounds it: the filters' issue
+// 3.0 ms; k = 64, L = 512: 250 and 180 us.  What bounds it: the filters' issue
 // latency (about five cycles per instruction and warp, two filter warps per SM
 // sub-partition at most), not the tensor pipe.
 //
