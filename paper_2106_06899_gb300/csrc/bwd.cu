@@ -44,6 +44,12 @@ struct __align__(16) BwdEntry {
   int key;   // bucket: (b, h) flattened times Lk plus the key index j
 };
 
+// one 16-byte load
+__device__ __forceinline__ BwdEntry ld_entry(const BwdEntry* p) {
+  const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+  return BwdEntry{static_cast<int>(u.x), __uint_as_float(u.y), __uint_as_float(u.z), static_cast<int>(u.w)};
+}
+
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -97,22 +103,37 @@ __device__ __forceinline__ void load_f32(const float* p, float (&f)[N]) {
   }
 }
 
-// the same columns of a dout row, which may be bf16 or fp32
-template <typename TD, int N>
-__device__ __forceinline__ void load_cols(const TD* p, float (&f)[N]) {
-  if constexpr (sizeof(TD) == 4) {
-    load_f32<N>(reinterpret_cast<const float*>(p), f);
-  } else {
-    static_assert(N % 8 == 0, "bf16 columns come in 16-byte chunks");
+// N columns of T as they lie in memory: rows in flight take half the registers
+// of widened ones
+template <typename T, int N>
+struct RawCols {
+  static constexpr int W = N * static_cast<int>(sizeof(T)) / 16;
+  uint4 u[W];
+  __device__ __forceinline__ void load(const T* p) {
 #pragma unroll
-    for (int i = 0; i < N / 8; ++i) {
-      float g[8];
-      Chunk<__nv_bfloat16>::load(reinterpret_cast<const __nv_bfloat16*>(p) + 8 * i, g);
+    for (int i = 0; i < W; ++i) u[i] = __ldg(reinterpret_cast<const uint4*>(p) + i);
+  }
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) f[8 * i + e] = g[e];
+    for (int i = 0; i < W; ++i) u[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  // acc += w * columns
+  __device__ __forceinline__ void add_to(float w, float (&acc)[N]) const {
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const uint32_t x[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if constexpr (sizeof(T) == 4) {
+          acc[4 * i + e] = fmaf(w, __uint_as_float(x[e]), acc[4 * i + e]);
+        } else {
+          acc[8 * i + 2 * e] = fmaf(w, __uint_as_float(x[e] << 16), acc[8 * i + 2 * e]);
+          acc[8 * i + 2 * e + 1] = fmaf(w, __uint_as_float(x[e] & 0xffff0000u), acc[8 * i + 2 * e + 1]);
+        }
+      }
     }
   }
-}
+};
 
 // ---------------------------------------------------------------------------
 // 1. rank
@@ -340,11 +361,12 @@ __global__ void __launch_bounds__(kRowWarps * 32) attn_bwd_rows_kernel(
 //        part[chunk][token][t];
 //   dx:  per (chunk, token) ds_t = sum over chunks of part (0 unless s_t > 0,
 //        ReLU's backward), then dx_i = sum_t ds_t W1_{j_t} over the chunk's
-//        columns (each thread 4 columns, 8 rows in flight); the chunk-0 CTA
+//        columns (each lane 8 columns, 8 rows in flight; 130 us with 4 columns
+//        per thread and 85 with 8 at 2048 x 1024 x 16384, k = 256: issue-bound); the chunk-0 CTA
 //        of a token also writes its entries to their key buckets.
 constexpr int kFfChunk = 256;
 constexpr int kDaWarps = 8;
-constexpr int kDxThreads = kFfChunk / 4;
+constexpr int kDxThreads = kFfChunk / 8;
 
 __global__ void __launch_bounds__(kDaWarps * 32) ffn_bwd_da_kernel(
     const __nv_bfloat16* __restrict__ W2, const float* __restrict__ dout, const int32_t* __restrict__ idx,
@@ -392,8 +414,7 @@ __global__ void __launch_bounds__(kDxThreads) ffn_bwd_dx_kernel(
     const __nv_bfloat16* __restrict__ W1, const int32_t* __restrict__ idx, const float* __restrict__ score,
     const float* __restrict__ part, const int* __restrict__ rank, const int* __restrict__ off,
     BwdEntry* __restrict__ ent, float* __restrict__ dx, int N, int DM, int dff, int K, int nchunks) {
-  extern __shared__ float dsv[];  // [K] ds_t, then [K] key indices (as int)
-  int* jv = reinterpret_cast<int*>(dsv + K);
+  extern __shared__ uint2 dsj[];  // [K] ds_t (bits) and key index, -1 if unused
   const int i = blockIdx.x % N, chunk = blockIdx.x / N;
   const int tid = threadIdx.x;
   for (int t = tid; t < K; t += kDxThreads) {
@@ -403,8 +424,7 @@ __global__ void __launch_bounds__(kDxThreads) ffn_bwd_dx_kernel(
     float ds = 0.f;
     if (use)
       for (int c = 0; c < nchunks; ++c) ds += part[(static_cast<long long>(c) * N + i) * K + t];
-    dsv[t] = ds;
-    jv[t] = use ? j : -1;
+    dsj[t] = make_uint2(__float_as_uint(ds), static_cast<uint32_t>(use ? j : -1));
     if (chunk == 0 && use) {  // this token's entries go to their key buckets once
       BwdEntry en;
       en.row = i;
@@ -415,29 +435,33 @@ __global__ void __launch_bounds__(kDxThreads) ffn_bwd_dx_kernel(
     }
   }
   __syncthreads();
-  const int c0 = chunk * kFfChunk + tid * 4;
+  const int c0 = chunk * kFfChunk + tid * 8;
   if (c0 >= DM) return;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   for (int t0 = 0; t0 < K; t0 += 8) {
-    uint2 raw[8];
+    uint4 raw[8];
     float w[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int t = t0 + u;
-      const int j = t < K ? jv[t] : -1;
-      w[u] = j >= 0 ? dsv[t] : 0.f;
-      raw[u] = j >= 0 ? __ldg(reinterpret_cast<const uint2*>(W1 + static_cast<long long>(j) * DM + c0))
-                      : make_uint2(0u, 0u);
+      const uint2 e = t0 + u < K ? dsj[t0 + u] : make_uint2(0u, 0xffffffffu);
+      const int j = static_cast<int>(e.y);
+      w[u] = __uint_as_float(e.x);
+      raw[u] = j >= 0 ? __ldg(reinterpret_cast<const uint4*>(W1 + static_cast<long long>(j) * DM + c0))
+                      : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      a0 = fmaf(w[u], __uint_as_float(raw[u].x << 16), a0);
-      a1 = fmaf(w[u], __uint_as_float(raw[u].x & 0xffff0000u), a1);
-      a2 = fmaf(w[u], __uint_as_float(raw[u].y << 16), a2);
-      a3 = fmaf(w[u], __uint_as_float(raw[u].y & 0xffff0000u), a3);
+      const uint32_t x[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[2 * i] = fmaf(w[u], __uint_as_float(x[i] << 16), acc[2 * i]);
+        acc[2 * i + 1] = fmaf(w[u], __uint_as_float(x[i] & 0xffff0000u), acc[2 * i + 1]);
+      }
     }
   }
-  *reinterpret_cast<float4*>(dx + static_cast<long long>(i) * DM + c0) = make_float4(a0, a1, a2, a3);
+  float4* dst = reinterpret_cast<float4*>(dx + static_cast<long long>(i) * DM + c0);
+  dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
 }
 
 // ---------------------------------------------------------------------------
@@ -454,12 +478,19 @@ constexpr int kKeyWarps = 8;
 constexpr int kRun = 64;
 
 template <typename T, typename TD, int LPR, int CPL>
-__global__ void __launch_bounds__(kKeyWarps * 32) bwd_keys_kernel(
+__global__ void __launch_bounds__(kKeyWarps * 32, sizeof(T) == 4 ? 3 : 2) bwd_keys_kernel(
     const T* __restrict__ q, const TD* __restrict__ dout, const BwdEntry* __restrict__ ent,
     const int* __restrict__ total_ptr, float* __restrict__ dk, float* __restrict__ dv, int D) {
   constexpr int VEC = Chunk<T>::N;
   constexpr int G = 32 / LPR;
   constexpr int U = CPL >= 4 ? 1 : 4 / CPL;
+  // The chain entry -> row load -> sum bounds the kernel: the next entries travel
+  // while the rows of these are summed, and rows stay as loaded until then, so that
+  // two blocks still share an SM (widened ones take 151 registers, and attn_bwd at
+  // H12 L8192 d64 k64 got slower).  295 -> 191 us there; FF 2048 x 1024 x 16384,
+  // k = 256: 335 -> 238.  With fp32 rows they would cost a block per SM (94 to 106
+  // registers instead of 80).
+  constexpr bool kAhead = sizeof(T) == 2;
   static_assert(LPR >= 1 && LPR <= 32 && 32 % LPR == 0, "a row spans 1..32 lanes of a group");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / LPR, c = lane % LPR;
@@ -503,25 +534,33 @@ __global__ void __launch_bounds__(kKeyWarps * 32) bwd_keys_kernel(
         for (int e = 0; e < VEC; ++e) ak[u][e] = av[u][e] = 0.f;
       }
     };
+    auto load_entries = [&](BwdEntry (&d)[U], long long e) {
+#pragma unroll
+      for (int i = 0; i < U; ++i) d[i] = e + i < s1 ? ld_entry(ent + e + i) : BwdEntry{0, 0.f, 0.f, -1};
+    };
+    BwdEntry en[U];
+    if constexpr (kAhead) load_entries(en, s0);
     for (long long e0 = s0; e0 < s1; e0 += U) {
-      BwdEntry en[U];
-      float fq[U][CPL][VEC], fg[U][CPL][VEC];
+      if constexpr (!kAhead) load_entries(en, e0);
+      RawCols<T, VEC> fq[U][CPL];
+      RawCols<TD, VEC> fg[U][CPL];
 #pragma unroll
       for (int i = 0; i < U; ++i) {
         const bool ok = e0 + i < s1;
-        en[i] = ok ? ent[e0 + i] : BwdEntry{0, 0.f, 0.f, -1};
 #pragma unroll
         for (int u = 0; u < CPL; ++u) {
           const int ch = ch0 + c + LPR * u;
           if (ok && ch < nch) {
-            Chunk<T>::load(q + static_cast<long long>(en[i].row) * D + ch * VEC, fq[i][u]);
-            load_cols<TD, VEC>(dout + static_cast<long long>(en[i].row) * D + ch * VEC, fg[i][u]);
+            fq[i][u].load(q + static_cast<long long>(en[i].row) * D + ch * VEC);
+            fg[i][u].load(dout + static_cast<long long>(en[i].row) * D + ch * VEC);
           } else {
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) fq[i][u][e] = fg[i][u][e] = 0.f;
+            fq[i][u].zero();
+            fg[i][u].zero();
           }
         }
       }
+      BwdEntry nx[U];
+      if constexpr (kAhead) load_entries(nx, e0 + U);
 #pragma unroll
       for (int i = 0; i < U; ++i) {
         if (e0 + i >= s1) break;
@@ -531,12 +570,14 @@ __global__ void __launch_bounds__(kKeyWarps * 32) bwd_keys_kernel(
           head_cut = false;
         }
 #pragma unroll
-        for (int u = 0; u < CPL; ++u)
+        for (int u = 0; u < CPL; ++u) {
+          fq[i][u].add_to(en[i].ds, ak[u]);
+          fg[i][u].add_to(en[i].a, av[u]);
+        }
+      }
+      if constexpr (kAhead) {
 #pragma unroll
-          for (int e = 0; e < VEC; ++e) {
-            ak[u][e] = fmaf(en[i].ds, fq[i][u][e], ak[u][e]);
-            av[u][e] = fmaf(en[i].a, fg[i][u][e], av[u][e]);
-          }
+        for (int i = 0; i < U; ++i) en[i] = nx[i];
       }
     }
     const bool tail_cut = s1 < E && ent[s1].key == cur;
