@@ -103,10 +103,13 @@ struct Layout {
     return c >= min_cap(topk) ? c : 0;
   }
   static bool fits(int topk) { return cap(topk) > 0; }
-  // Classes of the bound stretch (RowList): 2 k, or what the warp's memory holds.
+  // Classes of the bound stretch (RowList): 2 k, or what the warp's memory holds,
+  // in multiples of the slots that a tile takes at most (groups of four keys).
+  static constexpr int kTileSlots = N / 4;
   static int classes(int topk) {
-    return std::min((std::max(2 * topk, 16) + 15) & ~15,
-                    static_cast<int>(List::bytes(cap(topk)) / (kListStride * 4)) & ~15);
+    const int mem = static_cast<int>(List::bytes(cap(topk)) / (kListStride * 4));
+    const int want = std::max(2 * topk, 16) + kTileSlots - 1;
+    return std::min(want, mem) / kTileSlots * kTileSlots;
   }
   static size_t bytes(int topk) { return kFixed + buf_bytes(topk) + NJ * List::bytes(cap(topk)); }
 
@@ -115,6 +118,22 @@ struct Layout {
     return kPark ? static_cast<size_t>(grid) * (park_keys_per_cta(topk) * 8 + NJ * SL * 32 * 4) : 0;
   }
 };
+
+// How the bound pass sorts its nb key tiles of N keys into classes (RowList): the
+// tiles' maxima over groups of `group` keys go to slots 0 .. n - 1 in turn, N / group
+// of them per tile.  Groups of 64 keys, or as many fewer as leave a group per class.
+// n is a multiple of a tile's slots, so that a tile never writes past slot n - 1
+// (32 slots per tile at N = 128, group = 4), and of 16.
+struct BoundSplit {
+  int group, n;
+};
+__host__ __device__ constexpr BoundSplit bound_split(int N, int nb, int classes) {
+  int group = 64;
+  while (group > 4 && nb * N < group * classes) group >>= 1;
+  const int per = N / group, unit = per > 16 ? per : 16;
+  const int n = nb * per < classes ? nb * per : classes;
+  return BoundSplit{group, n & ~(unit - 1)};
+}
 
 // Waits for an mbarrier phase: every lane tries once, then lane 0 polls.  The
 // whole warp leaves together.
@@ -425,12 +444,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int lim_min = empty ? 0 : static_cast<int>(row_limit(bh, i0));  // smallest limit of the warp's rows
         const int nb = bound_tiles(bh, qt, t0, t1, empty);
         if (nb > 0) {
-          // groups of 64 keys, or as many fewer as leave a group per class
-          int group = 64;
-          while (group > 4 && nb * N < group * classes) group >>= 1;
-          const int M = min(classes, (nb * N / group) & ~15);
+          const BoundSplit split = bound_split(N, nb, classes);
+          const int group = split.group, M = split.n;
           list.bound_begin(M);
-          int slot = 0;  // M is a multiple of 16: a tile's slots do not wrap
+          int slot = 0;
           auto stretch = [&](auto g) {
             constexpr int G = decltype(g)::value;
             for (int i = 0; i < nb; ++i, ++acc_it) {
