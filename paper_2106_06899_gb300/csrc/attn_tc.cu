@@ -6,7 +6,9 @@ namespace topk {
 size_t attn_tc_bytes_d128(const AttnArgs& a, int num_sms);
 int attn_tc_d128(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st);
 
-bool attn_tc_supports(const AttnArgs& a) {
+// Types, head sizes and masks served here; whether the lists of topk entries
+// fit is the plan's answer (no scratch, no launch).
+static bool attn_tc_supports(const AttnArgs& a) {
   if (a.dtype != 1 || a.topk > kTcMaxK || a.mask) return false;  // bit masks run on the SIMT kernel
   return a.d == 64 || a.d == 128;
 }

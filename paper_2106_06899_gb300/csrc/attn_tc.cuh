@@ -764,9 +764,9 @@ int launch_merge(const AttnArgs& a, const uint2* part_keys, const int* part_n, i
 
 // What a kernel variant needs for a call.
 struct TcPlan {
-  int ru = 0, N = 0, parts = 1, n_units = 0, grid = 0;
-  size_t park = 0, bytes = 0;
-  bool fits = false;
+  int parts = 1, n_units = 0, grid = 0;
+  size_t park = 0, bytes = 0;  // of device scratch
+  bool fits = false;           // the lists of topk entries fit in shared memory
 };
 
 template <int D, typename IdxT, int RT, int RPU>
@@ -775,12 +775,12 @@ struct Variant {
 
   static TcPlan plan(const AttnArgs& a, int num_sms) {
     TcPlan p;
-    p.ru = RT * RPU;
-    p.N = L::N;
+    constexpr int RU = RT * RPU;
     p.fits = L::fits(a.topk);
     p.parts = RT == 1 ? tc_parts(a, num_sms, L::N, RPU) : 1;
-    p.n_units = a.B * a.H * ((a.Lq + p.ru - 1) / p.ru) * p.parts;
+    p.n_units = a.B * a.H * ((a.Lq + RU - 1) / RU) * p.parts;
     p.grid = p.n_units < num_sms ? p.n_units : num_sms;
+    if (!p.fits) return p;
     p.park = p.parts == 1 ? L::park_bytes(p.grid, a.topk) : 0;
     p.bytes = p.park + parts_bytes(a, p.parts);
     return p;
@@ -789,6 +789,7 @@ struct Variant {
   static int launch(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st) {
     const int BH = a.B * a.H;
     const TcPlan p = plan(a, num_sms);
+    if (!p.fits) return 0;
     CUtensorMap tmq, tmk;
     if (!make_tmap_bf16_3d(&tmq, a.q, D, a.Lq, BH, BM)) return -1;
     if (!make_tmap_bf16_3d(&tmk, a.k, D, a.Lk, BH, L::N)) return -1;
@@ -835,7 +836,8 @@ struct Variant {
   }
 };
 
-// Which variant serves a call: f is called with the Variant.
+// Which variant serves a call: f is called with the Variant, which may not fit
+// (TcPlan::fits); the call is then not served here.
 // - Two query tiles per unit share each key tile and give an SM eight filter
 //   warps, which is faster for long rows (L = 65536, k = 64: 18.4 ms against
 //   31.8; L = 16384: 2.3 against 2.9), but they leave the epilogue half the
@@ -859,17 +861,20 @@ auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
   return f(Variant<D, IdxT, 1, 32>{});
 }
 
+template <int D, typename F>
+auto with_variant(const AttnArgs& a, int num_sms, F&& f) {
+  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+}
+
 // The two calls of attn_tc.cu for one head size.
 template <int D>
 size_t tc_bytes(const AttnArgs& a, int num_sms) {
-  auto f = [&](auto v) { return decltype(v)::plan(a, num_sms).bytes; };
-  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+  return with_variant<D>(a, num_sms, [&](auto v) { return decltype(v)::plan(a, num_sms).bytes; });
 }
 
 template <int D>
 int tc_launch(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st) {
-  auto f = [&](auto v) { return decltype(v)::launch(a, ctl, num_sms, st); };
-  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+  return with_variant<D>(a, num_sms, [&](auto v) { return decltype(v)::launch(a, ctl, num_sms, st); });
 }
 
 }  // namespace

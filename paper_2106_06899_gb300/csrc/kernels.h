@@ -11,7 +11,8 @@
 namespace topk {
 
 constexpr int kSimtMaxK = 512;
-// tcgen05 attention path limit: what the lists of a 32-row unit hold in shared memory
+// tcgen05 attention path limit; where the lists of topk entries do not fit in
+// shared memory the call is not served there (attn_tc returns 0)
 constexpr int kTcMaxK = 512;
 
 struct AttnArgs {
@@ -52,7 +53,6 @@ struct FfnArgs {
 // 0 if it does not serve the given shape, -1 on a CUDA error.
 int attn_simt(const AttnArgs& a, int num_sms, cudaStream_t st);
 int attn_tc(const AttnArgs& a, const DevCtl& ctl, int num_sms, cudaStream_t st);
-bool attn_tc_supports(const AttnArgs& a);
 // Bytes of device scratch attn_tc needs for these arguments on a device with
 // num_sms SMs: the kernel hands each unit's candidates to its epilogue warps
 // through it (a fixed amount per CTA, nothing per query row), and key parts (small

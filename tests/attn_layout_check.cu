@@ -37,6 +37,29 @@ void bound_slots() {
   }
 }
 
+// Every variant that a call would launch has room for its lists; one that has not takes no scratch.
+template <int D>
+void picked() {
+  for (int Lk : {600, 65536, 65537, 1000000})
+    for (int Lq : {1, 130, 5000})
+      for (int k = 1; k <= kTcMaxK; ++k) {
+        AttnArgs a{};
+        a.B = 1, a.H = 8, a.Lq = Lq, a.Lk = Lk, a.d = D, a.topk = k, a.dtype = 1;
+        with_variant<D>(a, 152, [&](auto v) {
+          using V = decltype(v);
+          const TcPlan p = V::plan(a, 152);
+          const int cap = V::L::cap(k);
+          const bool room = cap >= V::L::min_cap(k) && V::L::bytes(k) <= V::L::kMaxSmem;
+          if (p.fits != room || (!p.fits && p.bytes > 0)) {
+            std::printf("D %d Lq %d Lk %d k %d: fits %d, %d list slots, %zu bytes of scratch\n", D, Lq, Lk, k, p.fits, cap,
+                        p.bytes);
+            ++bad;
+          }
+          return 0;
+        });
+      }
+}
+
 template <int D, typename IdxT>
 void check() {
   bound_slots<D, IdxT, 2, BM>();
@@ -52,6 +75,8 @@ int main() {
   check<64, uint32_t>();
   check<128, uint16_t>();
   check<128, uint32_t>();
+  picked<64>();
+  picked<128>();
   std::printf("%d violations\n", bad);
   return bad != 0;
 }
