@@ -43,6 +43,7 @@ namespace {
 
 constexpr int BM = 128;        // rows of an MMA tile
 constexpr int kThreads = 512;  // 4 control warps, 4 RT filter warps, the rest epilogue
+constexpr size_t kMaxSmem = 232448;  // shared memory that a CTA may ask for
 
 // D: head size; RT: query tiles per unit; RPU: query rows of a tile that
 // belong to the unit.  The MMA tile always has 128 rows; with RPU = 64 or 32
@@ -87,7 +88,6 @@ struct Layout {
   // work (a warp per row finds it faster than a filter's lockstep passes do).
   static constexpr int hand(int topk) { return (topk + 32 + 31) & ~31; }
   static constexpr size_t OFF_LIST = OFF_CTRL + CTRL_BYTES;
-  static constexpr size_t kMaxSmem = 232448;
   static constexpr size_t kFixed = 1024 + OFF_LIST;
 
   static constexpr int min_cap(int topk) { return (topk + kListSlack + 8 + 7) & ~7; }
@@ -620,6 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Key parts per query tile: split only grids that would leave at least half
 // the SMs idle (a few query tiles against many keys), into as many parts as
 // fill the SMs in one wave, each with at least 4 key tiles.
+constexpr int kMaxParts = 8;
 int tc_parts(const AttnArgs& a, int num_sms, int N, int ru) {
   const long long units = static_cast<long long>(a.B) * a.H * ((a.Lq + ru - 1) / ru);
   if (units * 2 > num_sms) return 1;
@@ -627,7 +628,7 @@ int tc_parts(const AttnArgs& a, int num_sms, int N, int ru) {
   const int nk_min = (kend_min + N - 1) / N;
   long long p = num_sms / units;
   p = std::min<long long>(p, nk_min / 4);
-  p = std::min<long long>(p, 8);
+  p = std::min<long long>(p, kMaxParts);
   return static_cast<int>(std::max<long long>(p, 1));
 }
 
@@ -648,7 +649,14 @@ int bound_divisor(const AttnArgs& a) {
   return a.Lq <= BM && key_bytes > 512e6 ? 4 : 1;
 }
 
+// Rows (warps) per block of the merge: eight, or what their candidates leave room
+// for (8 parts of k = 455 and more).
+constexpr size_t merge_row_bytes(int parts, int topk) { return static_cast<size_t>(parts) * topk * sizeof(uint2); }
 constexpr int kMergeWarps = 8;
+constexpr int merge_warps(int parts, int topk) {
+  const size_t fit = kMaxSmem / merge_row_bytes(parts, topk);
+  return fit < kMergeWarps ? static_cast<int>(fit) : kMergeWarps;
+}
 
 // Merges a row's `parts` kept lists (each the exact top k of its key range, in
 // index order, so their union holds the row's top k), one warp per row.  The
@@ -661,12 +669,12 @@ __global__ void __launch_bounds__(kMergeWarps * 32)
     attn_merge_kernel(const uint2* __restrict__ part_keys, const int* __restrict__ part_n, int parts, int BH, int Lq,
                       int Lk, int topk, const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out,
                       int32_t* __restrict__ idx, float* __restrict__ score) {
-  extern __shared__ uint2 mk_all[];  // [kMergeWarps][parts * topk]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  extern __shared__ uint2 mk_all[];  // [warps][parts * topk]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   uint2* mk = mk_all + static_cast<size_t>(warp) * parts * topk;
   const long long rows = static_cast<long long>(BH) * Lq;
-  for (long long r = static_cast<long long>(blockIdx.x) * kMergeWarps + warp; r < rows;
-       r += static_cast<long long>(gridDim.x) * kMergeWarps) {
+  for (long long r = static_cast<long long>(blockIdx.x) * warps + warp; r < rows;
+       r += static_cast<long long>(gridDim.x) * warps) {
     int P = 0;
     uint32_t hi = 0u, lo = 0xffffffffu;
     for (int p = 0; p < parts; ++p) {
@@ -748,15 +756,16 @@ __global__ void __launch_bounds__(kMergeWarps * 32)
 template <int D, int KPL>
 int launch_merge(const AttnArgs& a, const uint2* part_keys, const int* part_n, int parts, int num_sms,
                  cudaStream_t st) {
-  const size_t msmem = static_cast<size_t>(kMergeWarps) * parts * a.topk * sizeof(uint2);
+  const int warps = merge_warps(parts, a.topk);
+  const size_t msmem = warps * merge_row_bytes(parts, a.topk);
   auto merge = attn_merge_kernel<D, KPL>;
   if (msmem > 48 * 1024 &&
       cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(msmem)) != cudaSuccess)
     return -1;
   const long long rows = static_cast<long long>(a.B) * a.H * a.Lq;
-  long long mgrid = (rows + kMergeWarps - 1) / kMergeWarps;
+  long long mgrid = (rows + warps - 1) / warps;
   if (mgrid > 16LL * num_sms) mgrid = 16LL * num_sms;
-  merge<<<static_cast<unsigned>(mgrid), kMergeWarps * 32, msmem, st>>>(
+  merge<<<static_cast<unsigned>(mgrid), warps * 32, msmem, st>>>(
       part_keys, part_n, parts, a.B * a.H, a.Lq, a.Lk, a.topk, static_cast<const __nv_bfloat16*>(a.v),
       static_cast<__nv_bfloat16*>(a.out), a.idx, a.score);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;

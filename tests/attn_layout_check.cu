@@ -49,7 +49,7 @@ void picked() {
           using V = decltype(v);
           const TcPlan p = V::plan(a, 152);
           const int cap = V::L::cap(k);
-          const bool room = cap >= V::L::min_cap(k) && V::L::bytes(k) <= V::L::kMaxSmem;
+          const bool room = cap >= V::L::min_cap(k) && V::L::bytes(k) <= kMaxSmem;
           if (p.fits != room || (!p.fits && p.bytes > 0)) {
             std::printf("D %d Lq %d Lk %d k %d: fits %d, %d list slots, %zu bytes of scratch\n", D, Lq, Lk, k, p.fits, cap,
                         p.bytes);
@@ -58,6 +58,18 @@ void picked() {
           return 0;
         });
       }
+}
+
+// The merge of a call's key parts fits in shared memory.
+void merges() {
+  for (int parts = 2; parts <= kMaxParts; ++parts)
+    for (int k = 1; k <= kTcMaxK; ++k) {
+      const int w = merge_warps(parts, k);
+      if (w < 1 || w > kMergeWarps || w * merge_row_bytes(parts, k) > kMaxSmem) {
+        std::printf("merge of %d parts, k %d: %d warps\n", parts, k, w);
+        ++bad;
+      }
+    }
 }
 
 template <int D, typename IdxT>
@@ -77,6 +89,7 @@ int main() {
   check<128, uint32_t>();
   picked<64>();
   picked<128>();
+  merges();
   std::printf("%d violations\n", bad);
   return bad != 0;
 }
