@@ -49,7 +49,8 @@ constexpr size_t kMaxSmem = 232448;  // shared memory that a CTA may ask for
 // belong to the unit.  The MMA tile always has 128 rows; with RPU = 64 or 32
 // (RT = 1) only the first RPU of them are the unit's, so that one row's list
 // can hold several hundred keys.
-template <int D, typename IdxT, int RT, int RPU>
+// LONG: rows of more than 65,536 keys (rowlist.cuh).
+template <int D, bool LONG, int RT, int RPU>
 struct Layout {
   static_assert(RT == 1 || RPU == BM, "reduced-row units take one query tile");
   static constexpr int N = D == 64 ? 128 : 64;  // keys per tile: 16 KB of K
@@ -61,7 +62,7 @@ struct Layout {
   // eight leave lists so short that they prune all the time: 15.5).
   static constexpr int OFFER = D == 128 && RPU == BM ? 16 : 32;
   static constexpr int RECS = RT == 2 || (D == 128 && RPU == BM) ? 4 : 8;
-  using List = RowList<IdxT, RECS>;
+  using List = RowList<RECS, LONG>;
   static constexpr int NQ = RPU / 32;      // filter warps per query tile
   static constexpr int NJ = RT * NQ;       // filter warps in all
   static constexpr int NE = 12 - 4 * RT;   // epilogue warps
@@ -97,7 +98,7 @@ struct Layout {
   // less often but let their thresholds lag further behind).
   static int cap(int topk) {
     const int want = (5 * topk / 2 + 64 + 7) & ~7;
-    int c = static_cast<int>((kMaxSmem - kFixed) / NJ / (kListStride * (4 + sizeof(IdxT)))) & ~7;
+    int c = static_cast<int>((kMaxSmem - kFixed) / NJ / (kListStride * 6)) & ~7;
     while (c > 0 && kFixed + buf_bytes(topk) + NJ * List::bytes(c) > kMaxSmem) c -= 8;
     c = std::min(c, std::max(want, min_cap(topk)));
     return c >= min_cap(topk) ? c : 0;
@@ -190,14 +191,15 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, const
   }
 }
 
-template <int D, typename IdxT, int RT, int RPU>
+template <int D, bool LONG, int RT, int RPU>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                    const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out, int BH, int H, int Lq,
                    int Lk, int topk, int cap, int classes, int bound_den, int causal,
                    const int32_t* __restrict__ kv_len, int n_units, int parts, uint2* __restrict__ part_keys, int* __restrict__ part_n, int32_t* __restrict__ idx,
-                   float* __restrict__ score, uint2* __restrict__ park, int* __restrict__ park_n, DevCtl ctl) {
-  using L = Layout<D, IdxT, RT, RPU>;
+                   float* __restrict__ score, uint2* __restrict__ park, int* __restrict__ park_n, uint16_t* breaks,
+                   DevCtl ctl) {
+  using L = Layout<D, LONG, RT, RPU>;
   using List = typename L::List;
   constexpr int kOffer = L::OFFER;
   constexpr int N = L::N, S = L::S, R = L::R, NACC = L::NACC, NQ = L::NQ, NJ = L::NJ, NE = L::NE;
@@ -305,11 +307,25 @@ __global__ void __launch_bounds__(kThreads, 1)
     return nb * N >= 6 * topk ? nb : 0;
   };
 
-  // entry t of row r of filter warp `job`'s lists
-  auto list_at = [&](int job, int r, int t) {
+  // Rows of more than 65,536 keys: where a filter warp's break counts lie, and how
+  // many of them a unit's key tiles [t0, t1) leave.
+  constexpr int kStretch = 65536 / N;  // key tiles
+  auto breaks_of = [&](int job) {
+    return breaks + (static_cast<size_t>(blockIdx.x) * NJ + job) * ((Lk - 1) / 65536) * 32;
+  };
+  auto n_breaks = [&](int t0, int t1) { return (t1 - 1) / kStretch - t0 / kStretch; };
+
+  // entry t of row r of filter warp `job`'s lists, of a unit's key tiles [t0, t1)
+  auto list_at = [&](int job, int r, int t, int t0, int t1) {
     const uint32_t base = smem_u32(list_mem + job * List::bytes(cap)) + List::M::kRecBytes;
-    return make_uint2(__float_as_uint(lds_f32(base + t * kScStep + r * 4)),
-                      lds_idx<IdxT>(base + cap * kScStep + t * kIxStep<IdxT> + r * static_cast<uint32_t>(sizeof(IdxT))));
+    uint32_t j = lds_u16(base + cap * kScStep + t * kIxStep + r * 2);
+    if constexpr (LONG) {
+      const uint16_t* b = breaks_of(job) + r;
+      uint32_t hi = t0 / kStretch;
+      for (int e = n_breaks(t0, t1); e > 0; --e, b += 32) hi += t >= *b ? 1u : 0u;
+      j |= hi << 16;
+    }
+    return make_uint2(__float_as_uint(lds_f32(base + t * kScStep + r * 4)), j);
   };
 
   if (warp == 0) {
@@ -424,6 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t acc_it = 0;
       List list;
       list.bind(list_mem + job * List::bytes(cap), cap, topk);
+      if constexpr (LONG) list.brk.p = breaks_of(job) + lane;
       bool ok = true;
       uint32_t s = 0;  // units done
       for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++s) {
@@ -480,6 +497,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         list.begin(tau0);
         for (int kt = t0; kt < t1; ++kt, ++acc_it) {
+          if constexpr (LONG)
+            if (kt % kStretch == 0 && kt > t0) list.next_stretch();
           const int b = rt * NACC + acc_it % NACC;
           if (!warp_wait(&acc_full[b], (acc_it / NACC) & 1u, ctl, abort_flag)) {
             ok = false;
@@ -519,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const size_t prow0 = (static_cast<size_t>(part) * BH + bh) * Lq + i0;
           for (int r = 0; r < 32 && i0 + r < Lq; ++r) {
             const int n = __shfl_sync(0xffffffffu, list_n, r);
-            for (int t = lane; t < n; t += 32) part_keys[(prow0 + r) * topk + t] = list_at(job, r, t);
+            for (int t = lane; t < n; t += 32) part_keys[(prow0 + r) * topk + t] = list_at(job, r, t, t0, t1);
           }
           if (i_row < Lq) part_n[prow0 + lane] = list_n;
           __syncwarp();
@@ -534,7 +553,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           uint2* pk = park + slot * 32 * hand;
           for (int r = 0; r < 32; ++r) {
             const int n = __shfl_sync(0xffffffffu, list_n, r);
-            for (int t = lane; t < n; t += 32) pk[r * hand + t] = list_at(job, r, t);
+            for (int t = lane; t < n; t += 32) pk[r * hand + t] = list_at(job, r, t, t0, t1);
           }
           park_n[slot * 32 + lane] = list_n;
           __syncwarp();
@@ -557,6 +576,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x, ++s) {
       int bh, qt, part;
       decode(u, bh, qt, part);
+      int t0, t1;
+      bool empty;
+      tile_range(bh, qt, part, t0, t1, empty);
       for (int w = e; w < NJ * L::NS; w += NE) {
         const int job = w / L::NS, r0 = (w % L::NS) * L::RS;
         if (!wait_count(&pk_done[job], s + 1, ctl, abort_flag)) {
@@ -600,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint2* pk = park + (slot * 32 + r0 + r) * hand;
             go([pk](int t) { return __ldcg(pk + t); });
           } else {
-            go([&, r](int t) { return list_at(job, r0 + r, t); });
+            go([&, r](int t) { return list_at(job, r0 + r, t, t0, t1); });
           }
         }
         __syncwarp();
@@ -774,13 +796,13 @@ int launch_merge(const AttnArgs& a, const uint2* part_keys, const int* part_n, i
 // What a kernel variant needs for a call.
 struct TcPlan {
   int parts = 1, n_units = 0, grid = 0;
-  size_t park = 0, bytes = 0;  // of device scratch
+  size_t park = 0, parts_keys = 0, bytes = 0;  // of device scratch: parked lists, parts' lists, in all
   bool fits = false;           // the lists of topk entries fit in shared memory
 };
 
-template <int D, typename IdxT, int RT, int RPU>
+template <int D, bool LONG, int RT, int RPU>
 struct Variant {
-  using L = Layout<D, IdxT, RT, RPU>;
+  using L = Layout<D, LONG, RT, RPU>;
 
   static TcPlan plan(const AttnArgs& a, int num_sms) {
     TcPlan p;
@@ -791,7 +813,9 @@ struct Variant {
     p.grid = p.n_units < num_sms ? p.n_units : num_sms;
     if (!p.fits) return p;
     p.park = p.parts == 1 ? L::park_bytes(p.grid, a.topk) : 0;
-    p.bytes = p.park + parts_bytes(a, p.parts);
+    p.parts_keys = parts_bytes(a, p.parts);
+    p.bytes = p.park + p.parts_keys;
+    if (LONG) p.bytes += static_cast<size_t>(p.grid) * L::NJ * ((a.Lk - 1) / 65536) * 32 * sizeof(uint16_t);
     return p;
   }
 
@@ -805,7 +829,7 @@ struct Variant {
     // At least 120 KB so that a second CTA never shares the SM: each CTA takes
     // all TMEM columns it needs for its whole (persistent) lifetime.
     const size_t smem = std::max<size_t>(L::bytes(a.topk), 120 * 1024);
-    auto kern = attn_tc_kernel<D, IdxT, RT, RPU>;
+    auto kern = attn_tc_kernel<D, LONG, RT, RPU>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
         cudaSuccess)
       return -1;
@@ -829,7 +853,8 @@ struct Variant {
     kern<<<p.grid, kThreads, smem, st>>>(tmq, tmk, static_cast<const __nv_bfloat16*>(a.v),
                                          static_cast<__nv_bfloat16*>(a.out), BH, a.H, a.Lq, a.Lk, a.topk,
                                          L::cap(a.topk), L::classes(a.topk), bound_divisor(a), a.causal, a.kv_len,
-                                         p.n_units, p.parts, part_keys, part_n, a.idx, a.score, park, park_n, ctl);
+                                         p.n_units, p.parts, part_keys, part_n, a.idx, a.score, park, park_n,
+                                         LONG ? reinterpret_cast<uint16_t*>(ws + p.park + p.parts_keys) : nullptr, ctl);
     if (cudaGetLastError() != cudaSuccess) return -1;
     if (p.parts == 1) return 1;
     int rc;
@@ -855,24 +880,22 @@ struct Variant {
 //   selection is asked for (causal L = 8192, k = 64: 0.75 ms against 0.68).
 // - Else one query tile; and, for k beyond what 128 rows' lists can hold, units
 //   of 64 or 32 query rows.
-// Indices take 16 bits up to 65,536 keys.  Above, 32-bit ones let only one query
-// tile's lists fit at k = 64: 1.5 times as long as the heaps that the lists replaced.
-template <int D, typename IdxT, typename F>
+template <int D, bool LONG, typename F>
 auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
-  if constexpr (D == 64 && sizeof(IdxT) == 2) {
+  if constexpr (D == 64) {
     const long long units2 = static_cast<long long>(a.B) * a.H * ((a.Lq + 2 * BM - 1) / (2 * BM));
     const int keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk;
-    if (Layout<D, IdxT, 2, BM>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
-      return f(Variant<D, IdxT, 2, BM>{});
+    if (Layout<D, LONG, 2, BM>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
+      return f(Variant<D, LONG, 2, BM>{});
   }
-  if (Layout<D, IdxT, 1, BM>::fits(a.topk)) return f(Variant<D, IdxT, 1, BM>{});
-  if (Layout<D, IdxT, 1, 64>::fits(a.topk)) return f(Variant<D, IdxT, 1, 64>{});
-  return f(Variant<D, IdxT, 1, 32>{});
+  if (Layout<D, LONG, 1, BM>::fits(a.topk)) return f(Variant<D, LONG, 1, BM>{});
+  if (Layout<D, LONG, 1, 64>::fits(a.topk)) return f(Variant<D, LONG, 1, 64>{});
+  return f(Variant<D, LONG, 1, 32>{});
 }
 
 template <int D, typename F>
 auto with_variant(const AttnArgs& a, int num_sms, F&& f) {
-  return a.Lk <= 65536 ? with_variant_i<D, uint16_t>(a, num_sms, f) : with_variant_i<D, uint32_t>(a, num_sms, f);
+  return a.Lk <= 65536 ? with_variant_i<D, false>(a, num_sms, f) : with_variant_i<D, true>(a, num_sms, f);
 }
 
 // The two calls of attn_tc.cu for one head size.

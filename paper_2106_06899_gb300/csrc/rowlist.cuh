@@ -24,6 +24,13 @@
 // latency (about five cycles per instruction and warp, two filter warps per SM
 // sub-partition at most), not the tensor pipe.
 //
+// Indices take 16 bits.  Rows of more than 65,536 keys (LONG) also keep, per 65,536
+// keys after the first, how many entries of the list come before them (Breaks):
+// the list is in key order, so an entry's position gives the rest of its index.
+// With 32 bits in the list instead, two query tiles' lists do not fit at k = 64 and
+// no lists at all at d = 128, k > 462.  L = 131,072, k = 64, d = 64, two heads: 20.5
+// and 12.3 ms; 8,192 rows, 131,072 keys, d = 128, k = 128, four heads: 9.2 and 5.7.
+//
 // Layout: [slot][row] with a row stride of 33, so that a warp's lockstep passes
 // (one slot, 32 rows) and a row's list read by 32 lanes are both free of bank
 // conflicts.
@@ -69,67 +76,40 @@ __device__ __forceinline__ float lds_f32(uint32_t a) {
 __device__ __forceinline__ void sts_f32(uint32_t a, float x) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory");
 }
-template <typename IdxT>
-__device__ __forceinline__ uint32_t lds_idx(uint32_t a) {
-  if constexpr (sizeof(IdxT) == 2) {
-    unsigned short x;
-    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(a) : "memory");
-    return x;
-  } else {
-    uint32_t x;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
-    return x;
-  }
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  unsigned short x;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(a) : "memory");
+  return x;
 }
-template <typename IdxT>
-__device__ __forceinline__ void sts_idx(uint32_t a, uint32_t x) {
-  if constexpr (sizeof(IdxT) == 2)
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(static_cast<unsigned short>(x)) : "memory");
-  else
-    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t x) {
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(static_cast<unsigned short>(x)) : "memory");
 }
 
 // An entry (x, j) stored at as, ai where x passes thr (GE: x >= thr, else
 // x > thr), without a branch; as, ai step to the next slot.  The steps go to new
 // registers: a store reads its address late, and a predicated step in place
 // would wait for that (eight appends take 107 cycles instead of 151).
-template <typename IdxT, bool GE>
+template <bool GE>
 __device__ __forceinline__ void append_if(float x, float thr, uint32_t j, uint32_t& as, uint32_t& ai) {
-  if constexpr (sizeof(IdxT) == 2) {
-    if constexpr (GE)
-      asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ge.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
-          "@q st.shared.u16 [%1], %4;\n\t}" ::"r"(as),
-          "r"(ai), "f"(x), "f"(thr), "h"(static_cast<unsigned short>(j))
-          : "memory");
-    else
-      asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
-          "@q st.shared.u16 [%1], %4;\n\t}" ::"r"(as),
-          "r"(ai), "f"(x), "f"(thr), "h"(static_cast<unsigned short>(j))
-          : "memory");
-  } else {
-    if constexpr (GE)
-      asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ge.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
-          "@q st.shared.u32 [%1], %4;\n\t}" ::"r"(as),
-          "r"(ai), "f"(x), "f"(thr), "r"(j)
-          : "memory");
-    else
-      asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
-          "@q st.shared.u32 [%1], %4;\n\t}" ::"r"(as),
-          "r"(ai), "f"(x), "f"(thr), "r"(j)
-          : "memory");
-  }
+  if constexpr (GE)
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ge.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
+        "@q st.shared.u16 [%1], %4;\n\t}" ::"r"(as),
+        "r"(ai), "f"(x), "f"(thr), "h"(static_cast<unsigned short>(j))
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.f32 [%0], %2;\n\t"
+        "@q st.shared.u16 [%1], %4;\n\t}" ::"r"(as),
+        "r"(ai), "f"(x), "f"(thr), "h"(static_cast<unsigned short>(j))
+        : "memory");
   const bool p = GE ? x >= thr : x > thr;
   as += p ? 4u * kListStride : 0u;
-  ai += p ? static_cast<uint32_t>(sizeof(IdxT)) * kListStride : 0u;
+  ai += p ? 2u * kListStride : 0u;
 }
 
 constexpr uint32_t kScStep = kListStride * 4;  // bytes between a row's scores
-template <typename IdxT>
-constexpr uint32_t kIxStep = kListStride * sizeof(IdxT);
+constexpr uint32_t kIxStep = kListStride * 2;  // bytes between their indices
 
 // Entries of a list at or above x among slots 0 .. cr - 1 (cr > 0, pads are -inf),
 // counted in floats: the adds then run on the FMA pipe, next to the compares on
@@ -239,23 +219,50 @@ static __device__ __noinline__ Threshold list_threshold(uint32_t sc, int k, int 
 
 // Keeps the entries >= thr of slots 0 .. cr - 1, in order; returns the address
 // after the last one kept.
-template <typename IdxT>
 static __device__ __noinline__ uint32_t list_compact(uint32_t sc, uint32_t ix, int cr, float thr) {
   uint32_t ws = sc, wi = ix;
 #pragma unroll 1
-  for (int i = 0; i < cr; i += 8, sc += 8 * kScStep, ix += 8 * kIxStep<IdxT>) {
+  for (int i = 0; i < cr; i += 8, sc += 8 * kScStep, ix += 8 * kIxStep) {
     float s[8];
     uint32_t j[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       s[e] = lds_f32(sc + e * kScStep);
-      j[e] = lds_idx<IdxT>(ix + e * kIxStep<IdxT>);
+      j[e] = lds_u16(ix + e * kIxStep);
     }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) append_if<IdxT, true>(s[e], thr, j[e], ws, wi);
+    for (int e = 0; e < 8; ++e) append_if<true>(s[e], thr, j[e], ws, wi);
   }
   return ws;
 }
+
+// How many of a row's entries come before each further stretch of 65,536 keys
+// (device memory, [stretch][row]; p is the lane's column).  Nothing for rows of
+// one stretch.
+template <bool LONG>
+struct Breaks {};
+template <>
+struct Breaks<true> {
+  uint16_t* p;
+  int n;  // stretches begun after the unit's first
+
+  // The counts once the entries from thr on (of those equal to it the first eq)
+  // are all that is left of slots 0 .. cr - 1.
+  __device__ __forceinline__ void move(uint32_t sc, int cr, float thr, int eq) const {
+    int e = 0, next = p[0], w = 0;
+#pragma unroll 1
+    for (int i = 0; i < cr; ++i) {
+      while (next == i) {
+        p[e * 32] = static_cast<uint16_t>(w);
+        next = ++e < n ? p[e * 32] : -1;
+      }
+      const float s = lds_f32(sc + i * kScStep);
+      w += s > thr || (s == thr && eq > 0) ? 1 : 0;
+      eq -= s == thr ? 1 : 0;
+    }
+    for (; e < n; ++e) p[e * 32] = static_cast<uint16_t>(w);
+  }
+};
 
 // Drops entries that cannot be in the top k, keeping the list order: lists of
 // more than k + slack entries go down to between k and k + slack of them (ties
@@ -264,29 +271,34 @@ struct Pruned {
   int cnt;
   float tau;
 };
-template <typename IdxT>
-static __device__ __noinline__ Pruned list_prune(uint32_t sc, uint32_t ix, int k, int slack, int cnt, float tau0) {
+template <bool LONG>
+static __device__ __noinline__ Pruned list_prune(uint32_t sc, uint32_t ix, int k, int slack, int cnt, float tau0,
+                                                 Breaks<LONG> brk) {
   const bool active = cnt > k + slack;
   if (!__any_sync(0xffffffffu, active)) return Pruned{cnt, tau0};
   const Threshold th = list_threshold(sc, k, slack, cnt, tau0);
   int eq = th.eq;
   const int cr = (static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(cnt))) + 7) & ~7;
   const float thr = active ? th.tau : -INFINITY;
+  if constexpr (LONG) {
+    if (active && brk.n > 0) brk.move(sc, cr, thr, eq);
+    __syncwarp();
+  }
   uint32_t ws = sc;
   if (__all_sync(0xffffffffu, eq == 0x3fffffff)) {
-    ws = list_compact<IdxT>(sc, ix, cr, thr);
+    ws = list_compact(sc, ix, cr, thr);
   } else {  // some row keeps only the first of its entries equal to thr
     uint32_t wi = ix;
 #pragma unroll 1
     for (int i = 0; i < cr; ++i) {
       const float s = lds_f32(sc + i * kScStep);
-      const uint32_t j = lds_idx<IdxT>(ix + i * kIxStep<IdxT>);
+      const uint32_t j = lds_u16(ix + i * kIxStep);
       const bool is_eq = s == thr;
       if (s > thr || (is_eq && eq > 0)) {
         sts_f32(ws, s);
-        sts_idx<IdxT>(wi, j);
+        sts_u16(wi, j);
         ws += kScStep;
-        wi += kIxStep<IdxT>;
+        wi += kIxStep;
       }
       eq -= is_eq ? 1 : 0;
     }
@@ -296,33 +308,25 @@ static __device__ __noinline__ Pruned list_prune(uint32_t sc, uint32_t ix, int k
 
 // A record (a group's eight scores and its first key index) stored where its
 // maximum m passes tau, without a branch.
-template <typename IdxT, int HI>
+template <int HI>
 __device__ __forceinline__ void record_if(float m, float tau, const float* v, uint32_t j, uint32_t ra, uint32_t rx) {
-  if constexpr (sizeof(IdxT) == 2)
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.v4.f32 [%0], {%4, %5, %6, %7};\n\t"
-        "@q st.shared.v4.f32 [%0+%13], {%8, %9, %10, %11};\n\t@q st.shared.u16 [%1], %12;\n\t}" ::"r"(ra),
-        "r"(rx), "f"(m), "f"(tau), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]),
-        "f"(v[7]), "h"(static_cast<unsigned short>(j)), "n"(HI)
-        : "memory");
-  else
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.v4.f32 [%0], {%4, %5, %6, %7};\n\t"
-        "@q st.shared.v4.f32 [%0+%13], {%8, %9, %10, %11};\n\t@q st.shared.u32 [%1], %12;\n\t}" ::"r"(ra),
-        "r"(rx), "f"(m), "f"(tau), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]),
-        "f"(v[7]), "r"(j), "n"(HI)
-        : "memory");
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %2, %3;\n\t@q st.shared.v4.f32 [%0], {%4, %5, %6, %7};\n\t"
+      "@q st.shared.v4.f32 [%0+%13], {%8, %9, %10, %11};\n\t@q st.shared.u16 [%1], %12;\n\t}" ::"r"(ra),
+      "r"(rx), "f"(m), "f"(tau), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]),
+      "f"(v[7]), "h"(static_cast<unsigned short>(j)), "n"(HI)
+      : "memory");
 }
 __device__ __forceinline__ void lds_v4(uint32_t a, float& x, float& y, float& z, float& w) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x), "=f"(y), "=f"(z), "=f"(w) : "r"(a) : "memory");
 }
 
 // Where a warp's records and lists lie in its shared memory `mem`; lane r's row.
-// IdxT: uint16_t for up to 65,536 keys, else uint32_t.  R records per row.
-template <typename IdxT, int R>
+// R records per row.
+template <int R>
 struct ListMem {
   static constexpr uint32_t kRecStep = 512;  // bytes between a row's records
-  static constexpr uint32_t kRixStep = 32 * sizeof(IdxT);
+  static constexpr uint32_t kRixStep = 64;
   static constexpr uint32_t kRecHi = R * kRecStep;  // from a record's scores 0..3 to 4..7
   static constexpr uint32_t kRecBytes = 2 * R * kRecStep + R * kRixStep;
 
@@ -334,9 +338,9 @@ struct ListMem {
   __device__ __forceinline__ ListMem(uint32_t mem, int cap) {
     const uint32_t lane = threadIdx.x & 31;
     rec = mem + lane * 16;
-    rix = mem + 2 * R * kRecStep + lane * static_cast<uint32_t>(sizeof(IdxT));
+    rix = mem + 2 * R * kRecStep + lane * 2;
     sc = mem + kRecBytes + lane * 4;
-    ix = mem + kRecBytes + cap * kScStep + lane * static_cast<uint32_t>(sizeof(IdxT));
+    ix = mem + kRecBytes + cap * kScStep + lane * 2;
   }
 };
 
@@ -347,13 +351,14 @@ struct ListEnd {
   uint32_t as;
   float tau;
 };
-template <typename IdxT, int R>
-static __device__ __noinline__ ListEnd list_expand(uint32_t mem, int cap, int k, uint32_t ra, uint32_t as, float tau) {
-  using M = ListMem<IdxT, R>;
+template <int R, bool LONG>
+static __device__ __noinline__ ListEnd list_expand(uint32_t mem, int cap, int k, uint32_t ra, uint32_t as, float tau,
+                                                   Breaks<LONG> brk) {
+  using M = ListMem<R>;
   const M l(mem, cap);
   const int rc = static_cast<int>((ra - l.rec) / M::kRecStep);
   const int steps = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(rc)));
-  uint32_t ai = l.ix + (as - l.sc) / 4 * static_cast<uint32_t>(sizeof(IdxT));
+  uint32_t ai = l.ix + (as - l.sc) / 2;
   const uint32_t tight = l.sc + (cap - 8) * kScStep;
 #pragma unroll 1
   for (int i = 0; i < steps; ++i) {
@@ -361,7 +366,7 @@ static __device__ __noinline__ ListEnd list_expand(uint32_t mem, int cap, int k,
     const uint32_t a = l.rec + i * M::kRecStep;
     lds_v4(a, x[0], x[1], x[2], x[3]);
     lds_v4(a + M::kRecHi, x[4], x[5], x[6], x[7]);
-    const uint32_t j = lds_idx<IdxT>(l.rix + i * M::kRixStep);
+    const uint32_t j = lds_u16(l.rix + i * M::kRixStep);
     const bool live = i < rc;
     if (__any_sync(0xffffffffu, as > tight)) {
       const int n = static_cast<int>((as - l.sc) / kScStep);
@@ -369,15 +374,15 @@ static __device__ __noinline__ ListEnd list_expand(uint32_t mem, int cap, int k,
 #pragma unroll
       for (int e = 0; e < 8; ++e) pc += live && x[e] > tau ? 1 : 0;
       if (__any_sync(0xffffffffu, n + pc > cap)) {
-        const Pruned pr = list_prune<IdxT>(l.sc, l.ix, k, kListSlack, n, tau);
+        const Pruned pr = list_prune<LONG>(l.sc, l.ix, k, kListSlack, n, tau, brk);
         as = l.sc + pr.cnt * kScStep;
-        ai = l.ix + pr.cnt * kIxStep<IdxT>;
+        ai = l.ix + pr.cnt * kIxStep;
         tau = pr.tau;
       }
     }
     const float thr = live ? tau : INFINITY;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) append_if<IdxT, false>(x[e], thr, j + e, as, ai);
+    for (int e = 0; e < 8; ++e) append_if<false>(x[e], thr, j + e, as, ai);
   }
   return ListEnd{as, tau};
 }
@@ -390,19 +395,20 @@ static __device__ __noinline__ ListEnd list_expand(uint32_t mem, int cap, int k,
 // warp expands the records of all its rows in lockstep into the lists.  That keeps
 // the work on the path that every passing group takes, mostly for one lane out
 // of 32, to a few instructions.
-template <typename IdxT, int R>
+template <int R, bool LONG>
 struct RowList {
-  using M = ListMem<IdxT, R>;
+  using M = ListMem<R>;
   uint32_t mem;  // the warp's memory: records, then lists
   int cap;       // list slots, a multiple of 8, at least k + kListSlack + 8
   int k;
   uint32_t ra;   // where the next record goes
   uint32_t as;   // where the next entry's score goes
   float tau;     // at least k keys seen score >= tau (-inf until that is known)
+  Breaks<LONG> brk;
 
   // bytes of one warp's records and lists (a multiple of 16)
   __host__ __device__ static constexpr size_t bytes(int cap_) {
-    return M::kRecBytes + ((static_cast<size_t>(cap_) * kListStride * (4 + sizeof(IdxT)) + 15) & ~size_t(15));
+    return M::kRecBytes + ((static_cast<size_t>(cap_) * kListStride * 6 + 15) & ~size_t(15));
   }
 
   __device__ __forceinline__ void bind(const uint8_t* mem_, int cap_, int k_) {
@@ -413,6 +419,7 @@ struct RowList {
 
   // Empty lists under the threshold tau (+inf for a row that takes no part).
   __device__ __forceinline__ void begin(float tau_) {
+    if constexpr (LONG) brk.n = 0;
     ra = mem + (threadIdx.x & 31) * 16;
     as = M(mem, cap).sc;
     tau = tau_;
@@ -474,8 +481,8 @@ struct RowList {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       if (any[g]) {
-        const uint32_t rx = mem + 2 * R * M::kRecStep + (ra - mem) / (16 / sizeof(IdxT));
-        record_if<IdxT, static_cast<int>(M::kRecHi)>(m[g], t, v + 8 * g, j0 + 8 * g, ra, rx);
+        const uint32_t rx = mem + 2 * R * M::kRecStep + (ra - mem) / 8;
+        record_if<static_cast<int>(M::kRecHi)>(m[g], t, v + 8 * g, j0 + 8 * g, ra, rx);
         ra += m[g] > t ? M::kRecStep : 0u;
         if (R <= G && __any_sync(0xffffffffu, ra >= mem + R * M::kRecStep)) expand();
       }
@@ -484,17 +491,24 @@ struct RowList {
   }
 
   __device__ __forceinline__ void expand() {
-    const ListEnd r = list_expand<IdxT, R>(mem, cap, k, ra, as, tau);
+    const ListEnd r = list_expand<R, LONG>(mem, cap, k, ra, as, tau, brk);
     as = r.as;
     tau = r.tau;
     ra = mem + (threadIdx.x & 31) * 16;
+  }
+
+  // The next keys' indices are the first of another stretch of 65,536.
+  __device__ __forceinline__ void next_stretch() {
+    expand();
+    brk.p[brk.n * 32] = static_cast<uint16_t>(count());
+    ++brk.n;
   }
 
   // The unit's last records, then lists of at most k + slack entries.
   __device__ __forceinline__ void finish(int slack) {
     expand();
     const M l(mem, cap);
-    as = l.sc + list_prune<IdxT>(l.sc, l.ix, k, slack, count(), tau).cnt * kScStep;
+    as = l.sc + list_prune<LONG>(l.sc, l.ix, k, slack, count(), tau, brk).cnt * kScStep;
   }
 };
 
