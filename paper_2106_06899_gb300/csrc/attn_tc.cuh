@@ -49,19 +49,15 @@ constexpr size_t kMaxSmem = 232448;  // shared memory that a CTA may ask for
 // belong to the unit.  The MMA tile always has 128 rows; with RPU = 64 or 32
 // (RT = 1) only the first RPU of them are the unit's, so that one row's list
 // can hold several hundred keys.
-// LONG: rows of more than 65,536 keys (rowlist.cuh).
-template <int D, bool LONG, int RT, int RPU>
+// LONG: rows of more than 65,536 keys.  RECS: records per row (rowlist.cuh); which
+// of four and eight of them, and with how many scores per offer, see with_variant_i.
+template <int D, bool LONG, int RT, int RPU, int RECS>
 struct Layout {
   static_assert(RT == 1 || RPU == BM, "reduced-row units take one query tile");
   static constexpr int N = D == 64 ? 128 : 64;  // keys per tile: 16 KB of K
   static constexpr int S = RT == 2 || RPU < BM ? 2 : 3;  // K stages
   static constexpr int R = D / 64;  // 128-byte column blocks per row
-  // Scores per offer and records per row (rowlist.cuh).  Eight records where
-  // the lists leave room (k = 256: 3.0 ms against 3.5 with four at L = 8192),
-  // four beside two query tiles' lists and at d = 128 (k = 128, L = 16384: 8.9 ms;
-  // eight leave lists so short that they prune all the time: 15.5).
-  static constexpr int OFFER = D == 128 && RPU == BM ? 16 : 32;
-  static constexpr int RECS = RT == 2 || (D == 128 && RPU == BM) ? 4 : 8;
+  static constexpr int OFFER = RT == 1 && RECS == 4 ? 16 : 32;  // scores per offer
   using List = RowList<RECS, LONG>;
   static constexpr int NQ = RPU / 32;      // filter warps per query tile
   static constexpr int NJ = RT * NQ;       // filter warps in all
@@ -191,7 +187,7 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, const
   }
 }
 
-template <int D, bool LONG, int RT, int RPU>
+template <int D, bool LONG, int RT, int RPU, int RECS>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                    const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out, int BH, int H, int Lq,
@@ -199,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const int32_t* __restrict__ kv_len, int n_units, int parts, uint2* __restrict__ part_keys, int* __restrict__ part_n, int32_t* __restrict__ idx,
                    float* __restrict__ score, uint2* __restrict__ park, int* __restrict__ park_n, uint16_t* breaks,
                    DevCtl ctl) {
-  using L = Layout<D, LONG, RT, RPU>;
+  using L = Layout<D, LONG, RT, RPU, RECS>;
   using List = typename L::List;
   constexpr int kOffer = L::OFFER;
   constexpr int N = L::N, S = L::S, R = L::R, NACC = L::NACC, NQ = L::NQ, NJ = L::NJ, NE = L::NE;
@@ -800,9 +796,9 @@ struct TcPlan {
   bool fits = false;           // the lists of topk entries fit in shared memory
 };
 
-template <int D, bool LONG, int RT, int RPU>
+template <int D, bool LONG, int RT, int RPU, int RECS>
 struct Variant {
-  using L = Layout<D, LONG, RT, RPU>;
+  using L = Layout<D, LONG, RT, RPU, RECS>;
 
   static TcPlan plan(const AttnArgs& a, int num_sms) {
     TcPlan p;
@@ -829,7 +825,7 @@ struct Variant {
     // At least 120 KB so that a second CTA never shares the SM: each CTA takes
     // all TMEM columns it needs for its whole (persistent) lifetime.
     const size_t smem = std::max<size_t>(L::bytes(a.topk), 120 * 1024);
-    auto kern = attn_tc_kernel<D, LONG, RT, RPU>;
+    auto kern = attn_tc_kernel<D, LONG, RT, RPU, RECS>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
         cudaSuccess)
       return -1;
@@ -880,17 +876,26 @@ struct Variant {
 //   selection is asked for (causal L = 8192, k = 64: 0.75 ms against 0.68).
 // - Else one query tile; and, for k beyond what 128 rows' lists can hold, units
 //   of 64 or 32 query rows.
+// Eight records per row and 32 scores per offer, but two query tiles leave room
+// for four records.  At d = 128 the larger query and key tiles do so as well once
+// k is large: the lists there have to hold 1.5 k (k up to 90), or they prune all
+// the time, and four records with 16 scores per offer are the better split.
+// L = 8,192, H = 12, d = 128, four records and eight: k = 16: 1105 and 967 us,
+// k = 64: 1420 and 1222; L = 1,000, k = 100: 163 and 167.
 template <int D, bool LONG, typename F>
 auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
   if constexpr (D == 64) {
     const long long units2 = static_cast<long long>(a.B) * a.H * ((a.Lq + 2 * BM - 1) / (2 * BM));
     const int keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk;
-    if (Layout<D, LONG, 2, BM>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
-      return f(Variant<D, LONG, 2, BM>{});
+    if (Layout<D, LONG, 2, BM, 4>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
+      return f(Variant<D, LONG, 2, BM, 4>{});
+    if (Layout<D, LONG, 1, BM, 8>::fits(a.topk)) return f(Variant<D, LONG, 1, BM, 8>{});
+  } else {
+    if (2 * Layout<D, LONG, 1, BM, 8>::cap(a.topk) >= 3 * a.topk) return f(Variant<D, LONG, 1, BM, 8>{});
+    if (Layout<D, LONG, 1, BM, 4>::fits(a.topk)) return f(Variant<D, LONG, 1, BM, 4>{});
   }
-  if (Layout<D, LONG, 1, BM>::fits(a.topk)) return f(Variant<D, LONG, 1, BM>{});
-  if (Layout<D, LONG, 1, 64>::fits(a.topk)) return f(Variant<D, LONG, 1, 64>{});
-  return f(Variant<D, LONG, 1, 32>{});
+  if (Layout<D, LONG, 1, 64, 8>::fits(a.topk)) return f(Variant<D, LONG, 1, 64, 8>{});
+  return f(Variant<D, LONG, 1, 32, 8>{});
 }
 
 template <int D, typename F>

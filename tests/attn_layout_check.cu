@@ -12,9 +12,9 @@ int bad = 0;
 
 // Every number of bound tiles (until the split no longer changes): the slots that the tiles write, one
 // tile after the other, lie below the class count and inside the warp's memory, and there are more than k.
-template <int D, int RT, int RPU>
+template <int D, int RT, int RPU, int RECS>
 void bound_slots() {
-  using L = Layout<D, false, RT, RPU>;
+  using L = Layout<D, false, RT, RPU, RECS>;
   for (int k = 1; k <= kTcMaxK; ++k) {
     if (!L::fits(k)) continue;
     const int classes = L::classes(k);
@@ -28,8 +28,8 @@ void bound_slots() {
         slot = slot + per >= s.n ? 0 : slot + per;
       }
       if (top > s.n || s.n <= k || static_cast<size_t>(top) * kScStep > mem) {
-        std::printf("D %d RT %d RPU %d k %d: %d bound tiles write %d of %d slots, %zu bytes of memory\n", D, RT, RPU,
-                    k, nb, top, s.n, mem);
+        std::printf("D %d RT %d RPU %d RECS %d k %d: %d bound tiles write %d of %d slots, %zu bytes of memory\n", D, RT, RPU,
+                    RECS, k, nb, top, s.n, mem);
         ++bad;
         break;
       }
@@ -73,10 +73,11 @@ void merges() {
 
 template <int D>
 void check() {
-  bound_slots<D, 2, BM>();
-  bound_slots<D, 1, BM>();
-  bound_slots<D, 1, 64>();
-  bound_slots<D, 1, 32>();
+  bound_slots<D, 2, BM, 4>();
+  bound_slots<D, 1, BM, 4>();
+  bound_slots<D, 1, BM, 8>();
+  bound_slots<D, 1, 64, 8>();
+  bound_slots<D, 1, 32, 8>();
   picked<D>();
 }
 
