@@ -294,9 +294,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // unit are scored twice, first only for their group maxima, so that the main
   // pass starts with a threshold (RowList::bound_begin).  The second GEMM costs
   // less than the candidates it saves: bounds over a quarter, three quarters and
-  // all of the keys took 20.3, 19.3 and 18.4 ms at L = 65536, k = 64.  Where the
-  // keys come from device memory each time it covers a quarter of them
-  // (bound_den = 4, see bound_divisor()).  Fewer than 6 k keys give no useful bound.
+  // all of the keys took 20.3, 19.3 and 18.4 ms at L = 65536, k = 64.  Where rows have
+  // many keys per k it covers a share of them (bound_divisor()).  Fewer than
+  // 6 k keys give no useful bound.
   auto bound_tiles = [&](int bh, int qt, int t0, int t1, bool empty) {
     if (empty) return 0;
     const int nb = (min(t1, static_cast<int>(row_limit(bh, qt * RU)) / N) - t0) / bound_den;
@@ -656,15 +656,27 @@ size_t parts_bytes(const AttnArgs& a, int parts) {
   return static_cast<size_t>(parts) * rows * (static_cast<size_t>(a.topk) * 8 + 4);
 }
 
-// The share of the keys that the bound pass covers.  With one query tile per
-// head nobody else reads a head's keys; once they are several times what L2
-// holds (129 MB) a second pass over them reads device memory again.  Measured,
-// all of the keys against a quarter: 1.07 GB of keys (one position each,
-// d = 128) 589 and 433 us, 1.6 GB (128 positions) 1474 and 1312 us, but 0.40 GB
-// (128 positions, d = 64) 336 and 391 us.
-int bound_divisor(const AttnArgs& a) {
-  const double key_bytes = 2.0 * a.B * a.H * a.Lk * a.d;
-  return a.Lq <= BM && key_bytes > 512e6 ? 4 : 1;
+// The bound pass covers 1 / divisor of the keys.  A share f of n keys costs f n and
+// leaves about k / f candidates to append, so the best share goes with the root of
+// k / n: the divisor is the largest power of two up to sqrt(n / (k per)).  `per` is
+// smaller where a key of the bound pass costs more: at d = 128 (twice the MMA work),
+// and where every call reads the keys from device memory (few positions per head
+// against more keys than several times the 129 MB of L2).  At d = 64 lists of less
+// than 1.5 k slots prune for every few candidates, and there all of the keys pay.
+// us, all of the keys / the divisor's share:
+//   d = 64    131,072 keys, 2 heads, k = 16: 9242 / 7920 (4); k = 64: 12191, halved 13453
+//             16,384 keys, 1 head, k = 8: 233 / 219 (2); k = 32: 262, halved 269
+//   d = 128   8,192 keys, 12 heads, k = 1: 857 / 614 (8); k = 16: 967 / 878 (2)
+//             32,768 keys, 8 heads, causal, k = 128: 7134, halved 7453
+//   one position, 256 heads, 65,536 keys, d = 64, k = 16: 1391 / 850 (8); k = 128: 1488 / 1375 (2)
+int bound_divisor(const AttnArgs& a, int cap, int recs) {
+  const bool from_memory = a.Lq <= BM / 2 && 2.0 * a.B * a.H * a.Lk * a.d > 512e6;
+  if (!from_memory && a.d == 64 && 2 * cap < 3 * a.topk) return 1;
+  const int per = from_memory ? (a.d == 64 ? 40 : 16) : a.d == 64 ? 512 : recs == 8 ? 64 : 128;
+  const long long keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk;
+  int div = 1;
+  while (div < 16 && 4LL * div * div * per * a.topk <= keys) div *= 2;
+  return div;
 }
 
 // Rows (warps) per block of the merge: eight, or what their candidates leave room
@@ -848,7 +860,8 @@ struct Variant {
     }
     kern<<<p.grid, kThreads, smem, st>>>(tmq, tmk, static_cast<const __nv_bfloat16*>(a.v),
                                          static_cast<__nv_bfloat16*>(a.out), BH, a.H, a.Lq, a.Lk, a.topk,
-                                         L::cap(a.topk), L::classes(a.topk), bound_divisor(a), a.causal, a.kv_len,
+                                         L::cap(a.topk), L::classes(a.topk), bound_divisor(a, L::cap(a.topk), RECS),
+                                         a.causal, a.kv_len,
                                          p.n_units, p.parts, part_keys, part_n, a.idx, a.score, park, park_n,
                                          LONG ? reinterpret_cast<uint16_t*>(ws + p.park + p.parts_keys) : nullptr, ctl);
     if (cudaGetLastError() != cudaSuccess) return -1;
