@@ -820,10 +820,13 @@ struct Variant {
     p.n_units = a.B * a.H * ((a.Lq + RU - 1) / RU) * p.parts;
     p.grid = p.n_units < num_sms ? p.n_units : num_sms;
     if (!p.fits) return p;
-    p.park = p.parts == 1 ? L::park_bytes(p.grid, a.topk) : 0;
+    // for as many CTAs as units of one query tile would have: whether two share a
+    // unit may depend on what topk_attn_workspace_bytes() is not told
+    const int ctas = std::min(RT * p.n_units, num_sms);
+    p.park = p.parts == 1 ? L::park_bytes(ctas, a.topk) : 0;
     p.parts_keys = parts_bytes(a, p.parts);
     p.bytes = p.park + p.parts_keys;
-    if (LONG) p.bytes += static_cast<size_t>(p.grid) * L::NJ * ((a.Lk - 1) / 65536) * 32 * sizeof(uint16_t);
+    if (LONG) p.bytes += static_cast<size_t>(ctas) * L::NJ * ((a.Lk - 1) / 65536) * 32 * sizeof(uint16_t);
     return p;
   }
 
@@ -879,14 +882,31 @@ struct Variant {
   }
 };
 
+// Whether units of two query tiles are faster than units of one.  They share each
+// key tile and give an SM eight filter warps instead of four (L = 65,536, k = 64:
+// 18.4 ms against 31.8), but they leave the epilogue four warps for 256 rows instead
+// of eight for 128.  It has to keep up with the filters, so rows need 8,192 keys
+// (L = 4,096, k = 16, H = 12: 353 us against 263) and 128 k of them, twice that where
+// it also orders the selection (L = 16,384, causal, H = 8, k = 64: 1505 against 1328;
+// k = 32: 1036 against 1091).  And a grid of half the units, each 1.4 (from 512 k keys
+// on) to 1.6 times as long, has to end sooner: waves of units over the SMs are
+// compared (L = 8,192, k = 64, H = 6: three waves 517, two 609; L = 16,384, k = 16,
+// H = 3: three waves 654, two 537; 8,192 rows, 131,072 keys, k = 64, H = 4: 2729, 2085).
+bool two_query_tiles(const AttnArgs& a, int num_sms) {
+  const long long keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk, k = a.topk;
+  if (keys < 8192 || keys < (a.idx || a.score ? 256 : 128) * k) return false;
+  auto waves = [&](int rows) {
+    return (static_cast<long long>(a.B) * a.H * ((a.Lq + rows - 1) / rows) + num_sms - 1) / num_sms;
+  };
+  const long long w1 = waves(BM), w2 = waves(2 * BM);
+  if (w2 == 1 && keys < 256 * k) return false;  // 8,192 keys, k = 64, H = 4: 376 us against 358
+  return 5 * w1 > (keys >= 512 * k ? 7 : 8) * w2;
+}
+
 // Which variant serves a call: f is called with the Variant, which may not fit
 // (TcPlan::fits); the call is then not served here.
-// - Two query tiles per unit share each key tile and give an SM eight filter
-//   warps, which is faster for long rows (L = 65536, k = 64: 18.4 ms against
-//   31.8; L = 16384: 2.3 against 2.9), but they leave the epilogue half the
-//   warps and the rows half the memory: it is used where the lists fit (k up to
-//   68 at d = 64), the grid fills the SMs, rows have 128 k keys on average and no
-//   selection is asked for (causal L = 8192, k = 64: 0.75 ms against 0.68).
+// - Two query tiles per unit where their lists fit (d = 64, k up to 68) and
+//   two_query_tiles() says so.
 // - Else one query tile; and, for k beyond what 128 rows' lists can hold, units
 //   of 64 or 32 query rows.
 // Eight records per row and 32 scores per offer, but two query tiles leave room
@@ -898,9 +918,7 @@ struct Variant {
 template <int D, bool LONG, typename F>
 auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
   if constexpr (D == 64) {
-    const long long units2 = static_cast<long long>(a.B) * a.H * ((a.Lq + 2 * BM - 1) / (2 * BM));
-    const int keys = a.causal ? a.Lk - a.Lq / 2 : a.Lk;
-    if (Layout<D, LONG, 2, BM, 4>::fits(a.topk) && units2 >= num_sms && keys >= 128 * a.topk && !a.idx && !a.score)
+    if (Layout<D, LONG, 2, BM, 4>::fits(a.topk) && two_query_tiles(a, num_sms))
       return f(Variant<D, LONG, 2, BM, 4>{});
     if (Layout<D, LONG, 1, BM, 8>::fits(a.topk)) return f(Variant<D, LONG, 1, BM, 8>{});
   } else {

@@ -27,15 +27,15 @@ def test_units_of_fewer_rows(topk, Lk, causal):
 @pytest.mark.parametrize("topk", [65, 66, 68])
 def test_two_query_tiles_causal(topk):
     # rows 768 .. 1791 of each head lie in units of 5 to 8 bound tiles
-    B, H, L = 1, 3, 17536
+    B, H, L = 1, 4, 17536
     q, k, v = W.attention_inputs(B, H, L, L, 64, seed=820 + topk, dist="lowrank")
-    early = np.concatenate([h * L + np.arange(700, 1900, 9) for h in range(H)])
+    early = np.concatenate([h * L + np.arange(700, 1900, 12) for h in range(H)])
     rows = np.concatenate([early, W.sample_rows(B * H * L, 60, seed=topk).numpy()])
     _outputs_match(q, k, v, topk, np.unique(rows), causal=True)
 
 
 def test_two_query_tiles_key_counts():
-    B, H, Lq, Lk, d, topk = 4, 5, 2000, 8500, 64, 66
+    B, H, Lq, Lk, d, topk = 4, 9, 2000, 8500, 64, 66
     q, k, v = W.attention_inputs(B, H, Lq, Lk, d, seed=830)
     kv_len = np.array([700, 1100, 8500, 30], dtype=np.int32)
     out = T.attention(q.cuda(), k.cuda(), v.cuda(), topk, kv_len=torch.from_numpy(kv_len).cuda())
