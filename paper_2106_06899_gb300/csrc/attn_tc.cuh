@@ -14,11 +14,12 @@
 //                tcgen05.ld.red, which returns each group of eight together
 //                with its maximum, and keeps the row's candidates in its list
 //                (rowlist.cuh).  After the unit's last key tile it cuts the
-//                lists to the exact top k and hands them over.
-//   the rest     epilogue: a warp per row orders the kept keys if the
-//                selection is an output, applies the softmax over them and
-//                gathers the matching value rows (rowfinish.cuh), while the
-//                filters stream the next unit.
+//                lists to the top k, or near it (Layout::hand), and hands them
+//                over.
+//   the rest     epilogue: a warp per row makes the cut exact, orders the kept
+//                keys if the selection is an output, applies the softmax over
+//                them and gathers the matching value rows (rowfinish.cuh),
+//                while the filters stream the next unit.
 //
 // The score tile never leaves TMEM/registers: no [C x Lk] matrix is written
 // to device memory (Sec. 2.2 "Query chunking": memory O(C Lk) becomes
@@ -81,9 +82,16 @@ struct Layout {
   static constexpr uint32_t TMEM_COLS = RT * NACC * N;
   static constexpr int NBARS = 2 * S + 2 + 2 * RT * NACC + RT;
   static constexpr size_t CTRL_BYTES = (static_cast<size_t>(NBARS) * 8 + 8 + 2 * 8 * 4 + RPU * 4 + 127) & ~size_t(127);
-  // Candidates of a row that the epilogue takes at most: the exact top k is its
-  // work (a warp per row finds it faster than a filter's lockstep passes do).
-  static constexpr int hand(int topk) { return (topk + 32 + 31) & ~31; }
+  // Entries of a row that the filters hand over at most: the exact top k, or up to
+  // k + 63 candidates that the epilogue cuts (a warp per row).  Parked lists are cut by
+  // the filters, 32 rows in lockstep (B8 H12 L512 k = 64: 185 us against 153; B32 H12
+  // L128 k = 16: 129 against 89), but where rows are so long that the filters bound
+  // the kernel (L = 65,536, k = 64: 17.9 ms against 18.1).  Lists of large k that stay
+  // in place are cut by the epilogue: the filters wait for it anyhow (L = 8,192,
+  // k = 256: 3.0 ms against 5.4).
+  // The buffer has room for k + 63 in either case: its size does not depend on Lk.
+  static constexpr int hand_max(int topk) { return (topk + 63) & ~31; }
+  static constexpr int hand(int topk, int Lk) { return kPark && Lk < 32768 ? topk : hand_max(topk); }
   static constexpr size_t OFF_LIST = OFF_CTRL + CTRL_BYTES;
   static constexpr size_t kFixed = 1024 + OFF_LIST;
 
@@ -110,7 +118,7 @@ struct Layout {
   }
   static size_t bytes(int topk) { return kFixed + buf_bytes(topk) + NJ * List::bytes(cap(topk)); }
 
-  static constexpr size_t park_keys_per_cta(int topk) { return kPark ? static_cast<size_t>(NJ) * SL * 32 * hand(topk) : 0; }
+  static constexpr size_t park_keys_per_cta(int topk) { return kPark ? static_cast<size_t>(NJ) * SL * 32 * hand_max(topk) : 0; }
   static constexpr size_t park_bytes(int grid, int topk) {
     return kPark ? static_cast<size_t>(grid) * (park_keys_per_cta(topk) * 8 + NJ * SL * 32 * 4) : 0;
   }
@@ -191,7 +199,7 @@ template <int D, bool LONG, int RT, int RPU, int RECS>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
                    const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ out, int BH, int H, int Lq,
-                   int Lk, int topk, int cap, int classes, int bound_den, int causal,
+                   int Lk, int topk, int cap, int hand, int classes, int bound_den, int causal,
                    const int32_t* __restrict__ kv_len, int n_units, int parts, uint2* __restrict__ part_keys, int* __restrict__ part_n, int32_t* __restrict__ idx,
                    float* __restrict__ score, uint2* __restrict__ park, int* __restrict__ park_n, uint16_t* breaks,
                    DevCtl ctl) {
@@ -201,7 +209,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int N = L::N, S = L::S, R = L::R, NACC = L::NACC, NQ = L::NQ, NJ = L::NJ, NE = L::NE;
   constexpr uint32_t IDESC = idesc_bf16_f32(BM, N);
   constexpr int RU = RPU * RT;  // query rows per unit
-  const int hand = L::hand(topk);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -863,9 +870,9 @@ struct Variant {
     }
     kern<<<p.grid, kThreads, smem, st>>>(tmq, tmk, static_cast<const __nv_bfloat16*>(a.v),
                                          static_cast<__nv_bfloat16*>(a.out), BH, a.H, a.Lq, a.Lk, a.topk,
-                                         L::cap(a.topk), L::classes(a.topk), bound_divisor(a, L::cap(a.topk), RECS),
-                                         a.causal, a.kv_len,
-                                         p.n_units, p.parts, part_keys, part_n, a.idx, a.score, park, park_n,
+                                         L::cap(a.topk), L::hand(a.topk, a.Lk), L::classes(a.topk),
+                                         bound_divisor(a, L::cap(a.topk), RECS), a.causal, a.kv_len, p.n_units,
+                                         p.parts, part_keys, part_n, a.idx, a.score, park, park_n,
                                          LONG ? reinterpret_cast<uint16_t*>(ws + p.park + p.parts_keys) : nullptr, ctl);
     if (cudaGetLastError() != cudaSuccess) return -1;
     if (p.parts == 1) return 1;

@@ -36,3 +36,12 @@ def test_scratch_within_the_query(Lk, causal):
         T.topk_check()
         used, _ = T.topk_pool_usage()
         assert used <= need + 4096
+
+
+@pytest.mark.parametrize("Lk", [32767, 32768])
+@pytest.mark.parametrize("d,topk", [(64, 1), (64, 64), (64, 130), (128, 90), (128, 128)])
+def test_cut_in_the_filters_or_the_epilogue(Lk, d, topk):
+    # on both sides of the key count that says which; ties at the cut included
+    q, k, v = W.attention_inputs(1, 20, 1100, Lk, d, seed=1010 + topk)
+    k[:, :, 1::2] = k[:, :, ::2][:, :, : Lk // 2]
+    _selection_matches(q, k, v, topk, W.sample_rows(20 * 1100, 100, seed=topk).numpy())
