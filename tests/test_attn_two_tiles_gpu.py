@@ -23,6 +23,12 @@ def test_selection_and_outputs(topk, H, Lq, Lk, causal):
     _selection_matches(q, k, v, topk, rows, causal)
 
 
+@pytest.mark.parametrize("Lq,topk", [(1, 16), (3, 64), (128, 8)])
+def test_second_tile_empty(Lq, topk):
+    q, k, v = W.attention_inputs(10, 16, Lq, 8200, 64, seed=1005 + topk)
+    _outputs_match(q, k, v, topk, W.sample_rows(160 * Lq, 150, seed=topk).numpy(), causal=True)
+
+
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("Lk", [16384, 70000])
 def test_scratch_within_the_query(Lk, causal):
