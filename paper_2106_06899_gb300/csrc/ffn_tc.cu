@@ -148,10 +148,11 @@ struct RowCand {
   uint32_t stage;     // shared address of the warp's staging area
   int cap, cnt, k;
   bool hist_on;
+  bool low;           // L has risen to mn
   float base, width, inv_width;
   float L;            // this slice already holds k keys scoring >= L, all of lower index than
                       // any key still to come: a later key must beat L strictly
-  float mn, mx;       // spread of the first k candidates
+  float mn, mx;       // spread of the candidates until low is set
   int kp;             // ceil(k / slices)
   float Lp;           // valid lower bound of this slice's kp-th largest score
 
@@ -162,10 +163,15 @@ struct RowCand {
 
   // Raise L from the histogram (called between key tiles).
   __device__ __forceinline__ void refresh() {
+    if (!low && cnt >= k) {
+      // at least k candidates so far, every one of them >= mn.  The histogram says
+      // nothing of a row whose scores are all in its lowest bins: without this a row
+      // of equal scores (an all-zero token) would append every key.
+      L = fmaxf(L, mn);
+      low = true;
+    }
     if (!hist_on) {
       if (cnt < k) return;
-      // at least k candidates so far, every one of them >= mn
-      L = fmaxf(L, mn);
       set_bins();
       hist[0] = static_cast<uint32_t>(cnt - 1);
       hist[bin(mx) * BM] += 1u;
@@ -210,8 +216,8 @@ struct RowCand {
   // Offer 32 scores (key indices j0 .. j0 + 31, m[g] the maximum of their g-th
   // eight): a score qualifies if it reaches the shared bound and beats the
   // slice's own bound strictly (see L above), which is one compare with T.  The
-  // list has room (see the caller).  FIRST: some lane of the warp has no
-  // histogram yet and tracks its candidates' spread.
+  // list has room (see the caller).  FIRST: some lane of the warp has fewer than k
+  // candidates yet and tracks their spread.
   //
   // The scores go to the warp's staging area in shared memory ([score / 4][row]
   // vectors), each lane forms the mask of its qualifying ones, and the warp walks
@@ -496,6 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const size_t row_stride = static_cast<size_t>(n_sl) * cap;
       rc.cnt = 0;
       rc.hist_on = false;
+      rc.low = false;
       rc.base = 0.0f;
       rc.width = 1.0f;
       rc.inv_width = 1.0f;
@@ -523,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t below = ord_f32(Lg) - 1u;  // the largest score below Lg (below +0 comes -0, its equal)
         if (below == 0x7fffffffu) --below;
         const float T = row_ok ? fmaxf(Ls, shared_key ? unord_f32(below) : -INFINITY) : INFINITY;
-        const bool first = __any_sync(0xffffffffu, row_ok && !rc.hist_on);
+        const bool first = __any_sync(0xffffffffu, row_ok && !rc.low);
 #pragma unroll 1
         for (int c = 0; c < NT / 32; ++c) {
           float v[32], m[4];
