@@ -701,6 +701,17 @@ __global__ void __launch_bounds__(kFinalThreads)
     bad = 0;
   }
   __syncthreads();
+  // A row without a kept set (a NaN token has no k scores; lists that the first
+  // kernel never wrote after a timeout): the error word says so, the selection
+  // outputs read as empty, and the gather gets k keys of weight 0 to read.
+  auto no_kept_set = [&]() {
+    if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
+    for (int t = tid; t < topk; t += kFinalThreads) {
+      kept[static_cast<size_t>(row) * topk + t] = make_key(0.0f, 0u);
+      if (idx) idx[static_cast<size_t>(row) * topk + t] = -1;
+      if (score) score[static_cast<size_t>(row) * topk + t] = -INFINITY;
+    }
+  };
   const uint32_t tk = row_tau[row];
   const float L = tk ? unord_f32(tk) : -INFINITY;
   for (int sl = tid; sl < n_sl; sl += kFinalThreads) {
@@ -708,10 +719,7 @@ __global__ void __launch_bounds__(kFinalThreads)
     if (c < 0 || c > cap) bad = 1;  // never written: the first kernel stopped early (a timeout)
   }
   __syncthreads();
-  if (bad) {
-    if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-    return;
-  }
+  if (bad) return no_kept_set();
   // visit every candidate slot of the row; all threads iterate together.
   // Each thread loads kFinalVec 16-byte vectors (two candidates each) before
   // it visits any of them, so that many loads are in flight per thread (the
@@ -798,8 +806,7 @@ __global__ void __launch_bounds__(kFinalThreads)
   const int n_all = n_keys;
   bool direct = n_all <= kFinalMaxCand;
   if (n_all < topk) {  // fewer candidates than k: cannot happen unless the lists are inconsistent
-    if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-    return;
+    return no_kept_set();
   }
   if (direct) {
     // keys[0 .. topk) become the kept keys, best first.  Sorting costs
@@ -861,8 +868,7 @@ __global__ void __launch_bounds__(kFinalThreads)
     radix_digit(any, score_of, prefix, pmask, shifts[pass], dmasks[pass], remaining);
     const int digit = sh_digit, above = sh_above, count = sh_count;
     if (digit < 0) {  // fewer candidates than k: cannot happen unless the lists are inconsistent
-      if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-      return;
+      return no_kept_set();
     }
     prefix |= static_cast<uint32_t>(digit) << shifts[pass];
     pmask |= dmasks[pass] << shifts[pass];
@@ -879,8 +885,7 @@ __global__ void __launch_bounds__(kFinalThreads)
       __syncthreads();
       const int nc = n_keys;
       if (nc != kept_or_open || nc < topk) {
-        if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-        return;
+        return no_kept_set();
       }
       bitonic_desc(keys, nc);
       direct = true;  // keys[0 .. topk) are the kept keys, best first
@@ -901,8 +906,7 @@ __global__ void __launch_bounds__(kFinalThreads)
       for (int pass = 0; pass < 3; ++pass) {
         radix_digit(is_tie, inv_index, p2, m2, shifts[pass], dmasks[pass], rem2);
         if (sh_digit < 0) {
-          if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-          return;
+          return no_kept_set();
         }
         p2 |= static_cast<uint32_t>(sh_digit) << shifts[pass];
         m2 |= dmasks[pass] << shifts[pass];
@@ -919,8 +923,7 @@ __global__ void __launch_bounds__(kFinalThreads)
     });
     __syncthreads();
     if (n_keys != topk) {
-      if (tid == 0) atomicOr(ctl.error, kDevErrWorkspace);
-      return;
+      return no_kept_set();
     }
     bitonic_desc(keys, topk);
   }
