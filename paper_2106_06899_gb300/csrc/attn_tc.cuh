@@ -926,15 +926,24 @@ bool two_query_tiles(const AttnArgs& a, int num_sms) {
 // the time, and four records with 16 scores per offer are the better split.
 // L = 8,192, H = 12, d = 128, four records and eight: k = 16: 1105 and 967 us,
 // k = 64: 1420 and 1222; L = 1,000, k = 100: 163 and 167.
+// Units of 128 rows whose lists hold fewer than k + 16 entries (k = 137 to 140) pay
+// only for rows of 16 k keys: short ones have no bound pass, and every eighth entry
+// prunes (H = 12, k = 140: L = 300: 231 us against 93 with units of 64 rows, 2,048:
+// 466 against 349, 4,096: 852 against 957).
+template <typename L>
+bool lists_pay(const AttnArgs& a) {
+  return L::fits(a.topk) && (L::cap(a.topk) >= a.topk + 16 || (a.causal ? a.Lk - a.Lq / 2 : a.Lk) >= 16 * a.topk);
+}
+
 template <int D, bool LONG, typename F>
 auto with_variant_i(const AttnArgs& a, int num_sms, F&& f) {
   if constexpr (D == 64) {
     if (Layout<D, LONG, 2, BM, 4>::fits(a.topk) && two_query_tiles(a, num_sms))
       return f(Variant<D, LONG, 2, BM, 4>{});
-    if (Layout<D, LONG, 1, BM, 8>::fits(a.topk)) return f(Variant<D, LONG, 1, BM, 8>{});
+    if (lists_pay<Layout<D, LONG, 1, BM, 8>>(a)) return f(Variant<D, LONG, 1, BM, 8>{});
   } else {
     if (2 * Layout<D, LONG, 1, BM, 8>::cap(a.topk) >= 3 * a.topk) return f(Variant<D, LONG, 1, BM, 8>{});
-    if (Layout<D, LONG, 1, BM, 4>::fits(a.topk)) return f(Variant<D, LONG, 1, BM, 4>{});
+    if (lists_pay<Layout<D, LONG, 1, BM, 4>>(a)) return f(Variant<D, LONG, 1, BM, 4>{});
   }
   if (Layout<D, LONG, 1, 64, 8>::fits(a.topk)) return f(Variant<D, LONG, 1, 64, 8>{});
   return f(Variant<D, LONG, 1, 32, 8>{});
