@@ -279,9 +279,10 @@ int topk_ffn_fwd_noalloc(const void* x, const void* W1, const void* W2, void* ou
  *     to its epilogue warps through it: per CTA (one per SM, at most one per
  *     128-query tile) 16 x 32 rows of topk + 32 (rounded up to a multiple of
  *     32) entries of 8 bytes plus a count of 4, whatever Lq and Lk are: 60 MB on
- *     152 SMs at topk = 64; none where k is so large that the lists stay in
- *     shared memory.  Rows of more than 65,536 keys add up to 512 bytes per CTA
- *     for each further 65,536 keys.  Sized for the current device, or for 152
+ *     152 SMs at topk = 64.  None where k is so large that the lists stay in
+ *     shared memory, up to 65,536 keys; such calls, calls of a few positions that
+ *     split their keys, and any beyond 16 million keys take up to 512 bytes per
+ *     CTA for each further 65,536 keys.  Sized for the current device, or for 152
  *     SMs (a GB300) when no device is visible.
  *   - feed-forward: linear in N (see topk_ffn_fwd). */
 size_t topk_attn_workspace_bytes(int B, int H, int Lq, int Lk, int d, int topk, int chunk, int dtype);

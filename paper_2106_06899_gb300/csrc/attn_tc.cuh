@@ -89,9 +89,19 @@ struct Layout {
   // the kernel (L = 65,536, k = 64: 17.9 ms against 18.1).  Lists of large k that stay
   // in place are cut by the epilogue: the filters wait for it anyhow (L = 8,192,
   // k = 256: 3.0 ms against 5.4).
-  // The buffer has room for k + 63 in either case: its size does not depend on Lk.
+  // The buffer has room for hand_max entries per row in any case, so that its size does
+  // not depend on Lk; LONG rows give the last ones up for their break counts.
   static constexpr int hand_max(int topk) { return (topk + 63) & ~31; }
-  static constexpr int hand(int topk, int Lk) { return kPark && Lk < 32768 ? topk : hand_max(topk); }
+  static constexpr int hand(int topk, int Lk) {
+    if (!kPark) return hand_max(topk);
+    if (!LONG) return Lk < 32768 ? topk : hand_max(topk);
+    const int given = (breaks(Lk) + 4 * SL - 1) / (4 * SL);  // 8 SL bytes each, 2 per break
+    return hand_max(topk) - given > topk ? hand_max(topk) - given : topk;
+  }
+  static constexpr int breaks(int Lk) { return (Lk - 1) / 65536; }
+  static constexpr bool breaks_in_park(int topk, int Lk) {  // up to 16 million keys
+    return kPark && breaks(Lk) <= 4 * SL * (hand_max(topk) - hand(topk, Lk));
+  }
   static constexpr size_t OFF_LIST = OFF_CTRL + CTRL_BYTES;
   static constexpr size_t kFixed = 1024 + OFF_LIST;
 
@@ -314,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // many of them a unit's key tiles [t0, t1) leave.
   constexpr int kStretch = 65536 / N;  // key tiles
   auto breaks_of = [&](int job) {
-    return breaks + (static_cast<size_t>(blockIdx.x) * NJ + job) * ((Lk - 1) / 65536) * 32;
+    return breaks + (static_cast<size_t>(blockIdx.x) * NJ + job) * L::breaks(Lk) * 32;
   };
   auto n_breaks = [&](int t0, int t1) { return (t1 - 1) / kStretch - t0 / kStretch; };
 
@@ -811,7 +821,8 @@ int launch_merge(const AttnArgs& a, const uint2* part_keys, const int* part_n, i
 // What a kernel variant needs for a call.
 struct TcPlan {
   int parts = 1, n_units = 0, grid = 0;
-  size_t park = 0, parts_keys = 0, bytes = 0;  // of device scratch: parked lists, parts' lists, in all
+  size_t park = 0, bytes = 0;  // of device scratch: parked lists, in all
+  size_t breaks = 0;           // where in it the break counts begin
   bool fits = false;           // the lists of topk entries fit in shared memory
 };
 
@@ -831,9 +842,13 @@ struct Variant {
     // unit may depend on what topk_attn_workspace_bytes() is not told
     const int ctas = std::min(RT * p.n_units, num_sms);
     p.park = p.parts == 1 ? L::park_bytes(ctas, a.topk) : 0;
-    p.parts_keys = parts_bytes(a, p.parts);
-    p.bytes = p.park + p.parts_keys;
-    if (LONG) p.bytes += static_cast<size_t>(ctas) * L::NJ * ((a.Lk - 1) / 65536) * 32 * sizeof(uint16_t);
+    p.bytes = p.park + parts_bytes(a, p.parts);
+    if (LONG && p.parts == 1 && L::breaks_in_park(a.topk, a.Lk)) {
+      p.breaks = static_cast<size_t>(p.grid) * L::NJ * L::SL * 32 * L::hand(a.topk, a.Lk) * sizeof(uint2);
+    } else if (LONG) {
+      p.breaks = p.bytes;
+      p.bytes += static_cast<size_t>(ctas) * L::NJ * L::breaks(a.Lk) * 32 * sizeof(uint16_t);
+    }
     return p;
   }
 
@@ -873,7 +888,7 @@ struct Variant {
                                          L::cap(a.topk), L::hand(a.topk, a.Lk), L::classes(a.topk),
                                          bound_divisor(a, L::cap(a.topk), RECS), a.causal, a.kv_len, p.n_units,
                                          p.parts, part_keys, part_n, a.idx, a.score, park, park_n,
-                                         LONG ? reinterpret_cast<uint16_t*>(ws + p.park + p.parts_keys) : nullptr, ctl);
+                                         LONG ? reinterpret_cast<uint16_t*>(ws + p.breaks) : nullptr, ctl);
     if (cudaGetLastError() != cudaSuccess) return -1;
     if (p.parts == 1) return 1;
     int rc;

@@ -59,6 +59,37 @@ void picked() {
       }
 }
 
+// The break counts of long rows lie inside the scratch and apart from the lists and counts in it; where
+// lists are parked they take none of their own up to 16 million keys.
+template <int D>
+void breaks() {
+  for (int Lk : {65537, 131072, 131073, 1 << 20, 16000000, 40000000})
+    for (int Lq : {1, 200, 9000, 40000})
+      for (int k = 1; k <= kTcMaxK; ++k) {
+        AttnArgs a{};
+        a.B = 1, a.H = 8, a.Lq = Lq, a.Lk = Lk, a.d = D, a.topk = k, a.dtype = 1;
+        with_variant<D>(a, 152, [&](auto v) {
+          using V = decltype(v);
+          using L = typename V::L;
+          const TcPlan p = V::plan(a, 152);
+          const size_t need = static_cast<size_t>(p.grid) * L::NJ * L::breaks(Lk) * 64, end = p.breaks + need;
+          const size_t keys = static_cast<size_t>(p.grid) * L::NJ * L::SL * 32 * L::hand(k, Lk) * 8;
+          bool ok = end <= p.bytes && L::hand(k, Lk) >= k;
+          if (p.park > 0)
+            ok = ok && ((p.breaks >= keys && end <= p.grid * L::park_keys_per_cta(k) * 8) || p.breaks >= p.park) &&
+                 (p.bytes == p.park || Lk > 16000000);
+          else
+            ok = ok && p.breaks >= parts_bytes(a, p.parts);
+          if (!ok) {
+            std::printf("D %d Lq %d Lk %d k %d: breaks at %zu .. %zu of %zu bytes, lists %zu, parked %zu\n", D, Lq, Lk, k,
+                        p.breaks, end, p.bytes, keys, p.park);
+            ++bad;
+          }
+          return 0;
+        });
+      }
+}
+
 // The merge of a call's key parts fits in shared memory.
 void merges() {
   for (int parts = 2; parts <= kMaxParts; ++parts)
@@ -79,6 +110,7 @@ void check() {
   bound_slots<D, 1, 64, 8>();
   bound_slots<D, 1, 32, 8>();
   picked<D>();
+  breaks<D>();
 }
 
 }  // namespace

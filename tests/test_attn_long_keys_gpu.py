@@ -64,3 +64,12 @@ def test_key_orders(Lq, order, topk):
     assert np.array_equal(idx.cpu().reshape(-1, topk).numpy()[rows], ref["idx"])
     assert (idx == idx[:, :, :1]).all()  # all query rows are the same
     assert np.abs(out.float().cpu().reshape(-1, d).numpy()[rows] - ref["out"]).max() <= 2e-2
+
+
+@pytest.mark.parametrize("d,topk", [(64, 64), (64, 100), (128, 33)])
+def test_a_million_keys(d, topk):
+    # 18 breaks per row, kept where the parked lists leave room for them
+    q, k, v = W.attention_inputs(1, 1, 10000, 1_200_000, d, seed=910 + topk)
+    rows = W.sample_rows(10000, 12, seed=topk).numpy()
+    _outputs_match(q, k, v, topk, rows)
+    _selection_matches(q, k, v, topk, rows)
