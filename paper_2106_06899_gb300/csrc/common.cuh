@@ -43,10 +43,6 @@ __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
@@ -126,51 +122,10 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ void st_release_u64(uint64_t* p, uint64_t v) {
-  asm volatile("st.release.cta.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v) : "memory");
-}
-
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
   return v;
-}
-
-__device__ __forceinline__ uint64_t ld_acquire_u64(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.acquire.cta.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
-  return v;
-}
-
-// Predicated shared-memory stores (no branch, no write when p is false).
-__device__ __forceinline__ void st_shared_u2_if(bool p, uint2* dst, uint32_t a, uint32_t b) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t"
-      "@q st.shared.v2.u32 [%1], {%2, %3};\n\t}" ::"r"(static_cast<int>(p)),
-      "r"(smem_u32(dst)), "r"(a), "r"(b)
-      : "memory");
-}
-
-// Predicated 64-bit store that also orders the compiler's memory accesses
-// around it (the same thread reads the slot back later).
-__device__ __forceinline__ void st_shared_u64_if(bool p, uint64_t* dst, uint64_t v) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t"
-      "@q st.shared.u64 [%1], %2;\n\t}" ::"r"(static_cast<int>(p)),
-      "r"(smem_u32(dst)), "l"(v)
-      : "memory");
-}
-
-// Relaxed load: a value that only ever grows (a threshold), read without
-// ordering the surrounding accesses.
-__device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.cta.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)));
-  return v;
-}
-
-__device__ __forceinline__ void st_relaxed_u64(uint64_t* p, uint64_t v) {
-  asm volatile("st.relaxed.cta.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v));
 }
 
 // ---------------------------------------------------------------- TMA
@@ -418,17 +373,6 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
-}
-
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred = 0;
-  asm volatile(
-      "{\n\t.reg .b32 rx;\n\t.reg .pred px;\n\t"
-      "elect.sync rx|px, %1;\n\t"
-      "selp.b32 %0, 1, 0, px;\n\t}"
-      : "=r"(pred)
-      : "r"(0xffffffffu));
-  return pred != 0;
 }
 
 }  // namespace topk
