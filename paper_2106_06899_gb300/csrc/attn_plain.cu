@@ -55,7 +55,7 @@ struct PlainLayout {
 __device__ __forceinline__ bool warp_wait_p(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
                                             volatile int* abort_flag) {
   int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, ctl, abort_flag) ? 1 : 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait<false>(bar, parity, ctl, abort_flag) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
   return ok != 0;
 }

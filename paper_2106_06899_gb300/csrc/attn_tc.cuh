@@ -156,7 +156,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const 
                                           volatile int* abort_flag) {
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow(bar, parity, ctl, abort_flag) ? 1 : 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow<true>(bar, parity, ctl, abort_flag) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
   if (ok) (void)mbar_try_wait(bar, parity);  // every lane observes the completed phase
   return ok != 0;
@@ -906,7 +906,7 @@ struct Variant {
 
 // Whether units of two query tiles are faster than units of one.  They share each
 // key tile and give an SM eight filter warps instead of four (L = 65,536, k = 64:
-// 18.4 ms against 31.8), but they leave the epilogue four warps for 256 rows instead
+// 17.9 ms against 31.8), but they leave the epilogue four warps for 256 rows instead
 // of eight for 128.  It has to keep up with the filters, so rows need 8,192 keys
 // (L = 4,096, k = 16, H = 12: 353 us against 263) and 128 k of them, twice that where
 // it also orders the selection (L = 16,384, causal, H = 8, k = 64: 1505 against 1328;

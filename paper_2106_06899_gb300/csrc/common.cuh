@@ -91,12 +91,16 @@ __device__ __forceinline__ bool mbar_try_wait_for(uint64_t* bar, uint32_t parity
 // another thread of the CTA already gave up.  The polling loop is out of line
 // (mbar_wait_slow): each wait site holds one try and a call instead of the
 // loop, which keeps the kernels' unrolled pipelines small in the instruction
-// cache.
+// cache.  SUSPEND: a try may sleep for up to 10 us, which leaves the issue slots to
+// busy warps where many wait (attention, FF scores); its wake-up is late where two
+// warps hand tiles to and fro (plain attention, L = 65,536: 28.0 ms with, 25.1
+// without).
+template <bool SUSPEND>
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
                                                    volatile int* abort_flag) {
   const unsigned long long t0 = global_ns();
   for (uint32_t spin = 1;; ++spin) {
-    if (mbar_try_wait_for(bar, parity, 10000u)) return true;
+    if (SUSPEND ? mbar_try_wait_for(bar, parity, 10000u) : mbar_try_wait(bar, parity)) return true;
     if ((spin & 63u) == 0u) {
       if (*abort_flag) return false;
       if (global_ns() - t0 > ctl.wait_limit_ns) {
@@ -108,10 +112,11 @@ static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parit
   }
 }
 
+template <bool SUSPEND>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
                                           volatile int* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
-  return mbar_wait_slow(bar, parity, ctl, abort_flag);
+  return mbar_wait_slow<SUSPEND>(bar, parity, ctl, abort_flag);
 }
 
 // ---------------------------------------------------------------- CTA-scope

@@ -120,7 +120,7 @@ Plan make_plan(int N, int d_model, int d_ff, int topk, int num_sms) {
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const DevCtl& ctl,
                                           volatile int* abort_flag) {
   int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, ctl, abort_flag) ? 1 : 0;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait<true>(bar, parity, ctl, abort_flag) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
