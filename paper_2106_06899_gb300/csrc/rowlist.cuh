@@ -18,18 +18,22 @@
 // dependent chain of about 150 instructions that the warp's lanes rarely share.
 // Here a bound taken from group maxima in a first pass over the keys (RowList)
 // leaves about 1.4 k candidates per row, each of them an append.  Measured,
-// heaps and lists: k = 64, L = 65,536, d = 64: 19.7 and 18.4 ms; k = 128,
-// L = 16,384 causal, d = 128: 15.8 and 8.9 ms; k = 256, L = 8,192: 11.3 and
-// 3.0 ms; k = 64, L = 512: 250 and 180 us.  What bounds it: the filters' issue
+// heaps and lists: k = 64, L = 65,536, d = 64: 19.7 and 17.9 ms; k = 128,
+// L = 16,384 causal, d = 128: 15.8 and 8.8 ms; k = 256, L = 8,192: 11.3 and
+// 3.0 ms; k = 64, L = 512: 250 and 165 us.  What bounds it: the filters' issue
 // latency (about five cycles per instruction and warp, two filter warps per SM
-// sub-partition at most), not the tensor pipe.
+// sub-partition at most), not the tensor pipe.  Heaps were faster where one
+// filter warp per sub-partition meets few candidates: d = 64, one query tile per
+// unit, k up to 32 of more than 8,000 keys (128 positions against 65,536 keys,
+// k = 16: 256 and 308 us), and where scores rise along the keys (L = 8,192, k = 64:
+// 6.4 and 10.0 ms).
 //
 // Indices take 16 bits.  Rows of more than 65,536 keys (LONG) also keep, per 65,536
 // keys after the first, how many entries of the list come before them (Breaks):
 // the list is in key order, so an entry's position gives the rest of its index.
 // With 32 bits in the list instead, two query tiles' lists do not fit at k = 64 and
 // no lists at all at d = 128, k > 462.  L = 131,072, k = 64, d = 64, two heads: 20.5
-// and 12.3 ms; 8,192 rows, 131,072 keys, d = 128, k = 128, four heads: 9.2 and 5.7.
+// and 12.3 ms; 8,192 rows, 131,072 keys, d = 128, k = 128, four heads: 9.2 and 5.4.
 //
 // Layout: [slot][row] with a row stride of 33, so that a warp's lockstep passes
 // (one slot, 32 rows) and a row's list read by 32 lanes are both free of bank
